@@ -144,25 +144,17 @@ void move_finish(Ctx& c, Ctrl* ctrl);
 
 // ---------------------------------------------------------------- colour.cu
 struct JpBuffers {
-  int32_t* cnt;                 // [n] uncoloured higher-priority neighbour arcs
-  int32_t* list0;               // [list_cap] ready lists
-  int32_t* list1;
-  int64_t list_cap;
-  unsigned long long* rcount;   // [n + 64] per-round ready-list sizes
-  unsigned long long* bcount;   // [n + 64] per-round counts of vertices whose push is spread
-  int32_t* big;                 // [list_cap] those vertices
-  int64_t* big_cb;              // [list_cap] their first push chunk
-  int32_t* cown;                // [chunk_cap] big-list entry of each push chunk
-  int64_t chunk_cap;            // >= A / 256 + n
-  unsigned long long* ccount;   // [n + 64] per-round push-chunk counts
-  int64_t* boff;                // [n + 1] bitmap word offsets
-  unsigned* used;               // [used_cap] colour bitmaps, ceil((deg + 1) / 32) words per vertex
-  int64_t used_cap;             // >= A / 32 + n
-  unsigned long long* round;    // [4] current round, grid-barrier counter and generation
-  int64_t* tile_tmp;            // scan scratch
+  int4* rec;                  // [n] vertex records
+  int4* list0;                // [list_cap] ready lists
+  int4* list1;
+  int64_t list_cap;           // >= n + A / 32: the row chunks of one round
+  unsigned* used;             // [A / 32 + n] colour bitmaps
+  unsigned long long* state;  // [kJpStateWords] list sizes, barrier, results
 };
+constexpr int kJpStateWords = 16;
 // Jones-Plassmann colouring of g (self-loops ignored).  Returns the number of colours.
-// Uses ctrl->cnt[3, 4, 7]; synchronises the stream once per batch of rounds.
+// -1 on failure: *err, or h_pinned[3..7] = coloured, colours, listed, rounds, guard trips.
+// Synchronises the stream once.
 // In a batched run `seg` makes the priority hash the graph-local id.
 int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g_struct, const int32_t* perm, const int64_t* h_bucket_offs,
                   uint64_t seed, int32_t pass, int32_t* colour, const JpBuffers& jb, Ctrl* ctrl,

@@ -93,11 +93,11 @@ typedef struct {
                                     holds in flight (small graphs keep every class on its own).  The
                                     first iteration, where most vertices move, takes every class on
                                     its own */
-  int32_t wait_spins;            /* bound of the device-side waits (the colouring's grid barrier in
-                                    deterministic mode): polls of about 64 ns each before a waiting
-                                    block gives up (0 = built-in, about 0.3 s).  A wait that runs out
-                                    ends the kernel on every block and the call returns
-                                    LOUVAIN_ERR_TIMEOUT; the handle stays usable */
+  int32_t wait_spins;            /* bound of the device-side waits (the grid barriers of the colouring
+                                    and of the class steps in deterministic mode): polls of about
+                                    0.6 us each before a waiting block gives up (0 = built-in, about
+                                    5 s).  A wait that runs out ends the kernel on every block and
+                                    the call returns LOUVAIN_ERR_TIMEOUT; the handle stays usable */
   int32_t host_arcs;             /* 1: graphs whose arcs do not fit in HBM.  The super-vertex graphs'
                                     arc buffers (four of n_arcs entries) live in pinned host memory
                                     that the kernels read and write in place over NVLink-C2C, and

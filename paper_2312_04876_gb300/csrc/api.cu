@@ -15,7 +15,7 @@
 
 #include <unistd.h>
 
-#include "internal.cuh"
+#include "persist.cuh"
 
 using namespace lv;
 
@@ -37,7 +37,7 @@ struct Workspace {
   int64_t n_cap = -1, a_cap = -1;
   DevAlloc core;
   // per vertex
-  void *K0 = nullptr, *K = nullptr, *Sig = nullptr, *tot = nullptr;  // 8-byte accumulators
+  void *K0 = nullptr, *K = nullptr, *Sig = nullptr, *Sig2 = nullptr, *tot = nullptr;  // 8-byte accumulators
   int32_t *Cp = nullptr, *colour = nullptr, *csize = nullptr, *mv_from = nullptr, *mv_to = nullptr;
   int32_t *perm = nullptr, *cperm = nullptr, *occ = nullptr, *counts = nullptr, *cursor = nullptr;
   int32_t *cverts = nullptr;
@@ -46,6 +46,7 @@ struct Workspace {
   int64_t jlist_cap = 0;
   unsigned* jused = nullptr;
   unsigned long long* jstate = nullptr;
+  unsigned long long* swstate = nullptr;  // persistent class steps: barrier words and sums
   uint8_t* flags = nullptr;
   int64_t *newid = nullptr, *coff = nullptr, *cdeg = nullptr, *len = nullptr, *tile_tmp = nullptr;
   RowSet rows[2];
@@ -268,14 +269,16 @@ louvain_status ensure_workspace(louvain_handle h, int64_t n, int64_t a) {
   const int64_t n1 = nc + 1;
   bool ok = true;
   ok = ok && dalloc(h, d, (long long**)&ws.K0, n1) && dalloc(h, d, (long long**)&ws.K, n1) &&
-       dalloc(h, d, (long long**)&ws.Sig, n1) && dalloc(h, d, (long long**)&ws.tot, n1);
+       dalloc(h, d, (long long**)&ws.Sig, n1) && dalloc(h, d, (long long**)&ws.Sig2, n1) &&
+       dalloc(h, d, (long long**)&ws.tot, n1);
   ok = ok && dalloc(h, d, &ws.Cp, n1) && dalloc(h, d, &ws.colour, n1) && dalloc(h, d, &ws.csize, n1) &&
        dalloc(h, d, &ws.mv_from, n1) && dalloc(h, d, &ws.mv_to, n1) && dalloc(h, d, &ws.perm, n1) &&
        dalloc(h, d, &ws.cperm, n1) && dalloc(h, d, &ws.occ, n1) && dalloc(h, d, &ws.counts, n1) &&
        dalloc(h, d, &ws.cursor, n1) && dalloc(h, d, &ws.cverts, n1);
   ws.jlist_cap = ac / 32 + n1 + 64;
   ok = ok && dalloc(h, d, &ws.jrec, n1) && dalloc(h, d, &ws.jl0, ws.jlist_cap) && dalloc(h, d, &ws.jl1, ws.jlist_cap) &&
-       dalloc(h, d, &ws.jused, ac / 32 + n1 + 64) && dalloc(h, d, &ws.jstate, kJpStateWords);
+       dalloc(h, d, &ws.jused, ac / 32 + n1 + 64) && dalloc(h, d, &ws.jstate, kJpStateWords) &&
+       dalloc(h, d, &ws.swstate, kSweepStateWords);
   ok = ok && dalloc(h, d, &ws.flags, n1) && dalloc(h, d, &ws.dperm, n1) && dalloc(h, d, &ws.csz, n1);
   // giant plans: giant rows have > 4096 arcs, so there are at most A / 4097 of them; chunks of >= 512
   // arcs over their rows: <= gcap + A / 512; slices of >= 128 slots over tables of < 4 x the arcs:
@@ -577,7 +580,7 @@ template <class M>
 void enqueue_iteration(louvain_handle h, Ctx& c, const GraphView<typename M::w_t>& g, const PassState<M>& st,
                        const std::vector<ClassStep>& steps, const int32_t* glist, bool det, bool pruning,
                        GraphCtl* gc, int32_t n_graphs, bool streams, const int64_t* recs = nullptr,
-                       const int32_t* gbase = nullptr) {
+                       const int32_t* gbase = nullptr, bool finish = true) {
   Workspace& ws = h->ws;
   GraphView<typename M::w_t> gk = g;
   if (recs) gk.n = 0;
@@ -619,6 +622,7 @@ void enqueue_iteration(louvain_handle h, Ctx& c, const GraphView<typename M::w_t
       if (!streams) prof_end(h, c, kApply, pm);
     }
   }
+  if (!finish) return;
   if (gc) batch_finish<M>(c, ws.ctrl, gc, n_graphs);
   else move_finish<M>(c, ws.ctrl);
 }
@@ -629,10 +633,11 @@ void enqueue_iteration(louvain_handle h, Ctx& c, const GraphView<typename M::w_t
 template <class M>
 std::vector<int64_t> iteration_key(louvain_handle h, const Ctx& c, const GraphView<typename M::w_t>& g,
                                    const PassState<M>& st, const std::vector<ClassStep>& steps, const int64_t* recs,
-                                   const int32_t* gbase, bool det, bool pruning, GraphCtl* gc, int32_t n_graphs) {
+                                   const int32_t* gbase, bool det, bool pruning, GraphCtl* gc, int32_t n_graphs,
+                                   bool finish = true) {
   static_assert(sizeof(PassState<M>) % 8 == 0 && sizeof(GiantPlan) % 8 == 0, "pointer-only records");
   const Workspace& ws = h->ws;
-  std::vector<int64_t> k = {M::is_fp ? 1 : 0, det ? 1 : 0, pruning ? 1 : 0, n_graphs, (int64_t)(intptr_t)gc,
+  std::vector<int64_t> k = {M::is_fp ? 1 : 0, det ? 1 : 0, pruning ? 1 : 0, finish ? 1 : 0, n_graphs, (int64_t)(intptr_t)gc,
                             c.num_sms, c.lm_blocks_per_sm, c.giant_min, (int64_t)(intptr_t)ws.perm,
                             (int64_t)(intptr_t)gbase, (int64_t)(intptr_t)recs, (int64_t)(intptr_t)ws.desc,
                             (int64_t)(intptr_t)g.rbeg, (int64_t)(intptr_t)g.rend, (int64_t)(intptr_t)g.tg,
@@ -653,8 +658,25 @@ std::vector<int64_t> iteration_key(louvain_handle h, const Ctx& c, const GraphVi
   return k;
 }
 
+// Which steps a block could make more moves in than it keeps (sweep.cu): rows are dealt to `blocks`
+// blocks, a bucket's by groups of 4, 8, 32, 128, 512 and 1024 threads.
+bool step_is_wide(const ClassStep& cs, int64_t blocks) {
+  static const int64_t kGroups[kNumBuckets - 1] = {256, 128, 32, 8, 2, 1};
+  int64_t most = cs.g1 - cs.g0;
+  for (int b = 0; b < kNumBuckets - 1; b++) most += (cs.count[b] + blocks * kGroups[b] - 1) / (blocks * kGroups[b]) * kGroups[b];
+  return most > kSweepMoves;
+}
+
+// Arcs of a step, about (a typical row length per bucket).
+int64_t step_arcs(const ClassStep& cs) {
+  static const int64_t kArcs[kNumBuckets - 1] = {3, 9, 48, 256, 1024, 3000};
+  int64_t a = 12000 * (cs.g1 - cs.g0);
+  for (int b = 0; b < kNumBuckets - 1; b++) a += cs.count[b] * kArcs[b];
+  return a;
+}
+
 // Host image of the step records of `steps` (kStepWords each; the giant list offset from its base).
-void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64_t* out) {
+void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64_t* out, int64_t blocks = 0) {
   for (size_t k = 0; k < steps.size(); k++) {
     int64_t* r = out + k * kStepWords;
     std::memset(r, 0, sizeof(int64_t) * kStepWords);
@@ -668,6 +690,7 @@ void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64
     r[kStepGiant + 2] = cs.g1;
     r[kStepApply] = cs.apply_start;
     r[kStepApply + 1] = cs.apply_count;
+    r[kStepWide] = blocks > 0 && step_is_wide(cs, blocks) ? 1 : 0;
   }
 }
 
@@ -689,7 +712,7 @@ louvain_status capture_iteration(louvain_handle h, Ctx& c0, const GraphView<type
                                  const std::vector<ClassStep>& steps, const int32_t* glist, bool det, bool pruning,
                                  GraphCtl* gc, int32_t n_graphs, cudaGraphExec_t exclude, cudaGraphExec_t* exec,
                                  int64_t* launches, int32_t* instantiated, const int64_t* recs,
-                                 const int32_t* gbase, const std::vector<int64_t>& key) {
+                                 const int32_t* gbase, const std::vector<int64_t>& key, bool finish = true) {
   *exec = nullptr;
   if (!h->cap && cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess)
     return cuda_err(h, cudaGetLastError(), "capture stream creation");
@@ -714,7 +737,7 @@ louvain_status capture_iteration(louvain_handle h, Ctx& c0, const GraphView<type
   move_prepare();
   cudaError_t e = cudaStreamBeginCapture(c.s, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_err(h, e, "graph capture begin");
-  enqueue_iteration<M>(h, c, g, st, steps, glist, det, pruning, gc, n_graphs, true, recs, gbase);
+  enqueue_iteration<M>(h, c, g, st, steps, glist, det, pruning, gc, n_graphs, true, recs, gbase, finish);
   cudaGraph_t graph = nullptr;
   e = cudaStreamEndCapture(c.s, &graph);
   *launches = c.launches;
@@ -774,6 +797,92 @@ louvain_status capture_iteration(louvain_handle h, Ctx& c0, const GraphView<type
   }
   h->execs.push_back({*exec, nodes, ++h->exec_clock, *launches, key, h->call_seq});
   return LOUVAIN_OK;
+}
+
+// Scope of the persistent class steps by the arcs of a step, about (step_arcs): one block up to 2048
+// (2,855 vertices, 1,122 arcs a step, 228 steps: 2.9 ms a phase on a block, 3.5 on a cluster; 5,486 arcs
+// a step: 8.5 against 5.2), a cluster up to 8000 (14,325 arcs a step: 1.0 ms on a cluster, 0.8 on the
+// grid), else the grid.  A class of over 8 million arcs keeps its per-bucket launches, as do those
+// before it: there a barrier more or less is nothing, and a launch's blocks retire as they finish
+// (24M-vertex grid, pass 1: 8.9 ms against 12.0 in the persistent launch).
+constexpr int64_t kSweepCtaArcs = 2048, kSweepClusterArcs = 8000, kSweepWideArcs = 8000000;
+// The deterministic phase's iterations: classes [0, f) as captured per-class launches, the others in
+// one persistent launch (sweep.cu); with f = 0 that launch runs the whole phase.
+template <class M>
+louvain_status sweep_phase(louvain_handle h, Ctx& c, const GraphView<typename M::w_t>& g, const PassState<M>& st,
+                           const std::vector<ClassStep>& steps, const int32_t* glist, const louvain_params& p,
+                           GraphCtl* gc, int32_t n_graphs, int32_t* li, int64_t* moves, float* ms_graph,
+                           int32_t* graphs_new) {
+  Workspace& ws = h->ws;
+  const bool pruning = p.pruning != 0;
+  louvain_status s;
+  size_t f = 0;
+  int64_t arcs = 0, most = 0;
+  for (size_t k = 0; k < steps.size(); k++) {
+    const int64_t a = step_arcs(steps[k]);
+    if (a > kSweepWideArcs) {
+      f = k + 1;
+      arcs = most = 0;
+    } else {
+      arcs += a;
+      most = std::max(most, a);
+    }
+  }
+  const int64_t narrow = (int64_t)(steps.size() - f), avg = narrow > 0 ? arcs / narrow : 0;
+  Scope scope = kGrid;
+  if (avg <= kSweepCtaArcs && most <= 16 * kSweepCtaArcs) scope = kCta;
+  else if (avg <= kSweepClusterArcs && most <= 16 * kSweepClusterArcs) scope = kCluster;
+  const int64_t blocks = scope == kCta ? 1 : (scope == kCluster ? kClusterBlocks : c.num_sms);
+  const int64_t words = (int64_t)steps.size() * kStepWords;
+  if ((s = ensure_desc(h, words)) != LOUVAIN_OK) return s;
+  write_step_records(steps, glist - ws.glist, h->dpin, blocks);
+  cudaMemcpyAsync(ws.desc, h->dpin, (size_t)words * sizeof(int64_t), cudaMemcpyHostToDevice, c.s);
+  auto now = [] { return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count(); };
+  const double t0 = now();
+  cudaGraphExec_t exec = nullptr;
+  int64_t launches = 0;
+  int32_t n_new = 0;
+  if (f > 0) {
+    const std::vector<ClassStep> wide(steps.begin(), steps.begin() + (std::ptrdiff_t)f);
+    const bool finish = narrow == 0;
+    const std::vector<int64_t> key = iteration_key<M>(h, c, g, st, wide, ws.desc, ws.glist, true, pruning, gc, n_graphs, finish);
+    if (auto* x = find_exec(h, key)) {
+      exec = x->e;
+      launches = x->launches;
+    } else if ((s = capture_iteration<M>(h, c, g, st, wide, glist, true, pruning, gc, n_graphs, nullptr, &exec, &launches,
+                                         &n_new, ws.desc, ws.glist, key, finish)) != LOUVAIN_OK) {
+      return s;
+    }
+  }
+  if (ms_graph) *ms_graph = (float)(now() - t0);
+  if (graphs_new) *graphs_new = n_new;
+  const SweepPlan sw{ws.Sig2, ws.swstate, ws.desc + (int64_t)f * kStepWords, (int)narrow, f == 0, (int)scope};
+  for (int32_t enq = 0;;) {
+    // two iterations between host reads (one launch runs them all without wide classes)
+    for (int k = 0; k < 2 && enq < p.max_iterations; k++, enq++) {
+      if (exec) {
+        cudaGraphLaunch(exec, c.s);
+        c.launches += launches;
+      }
+      if (narrow > 0) {
+        const cudaError_t e = move_sweep<M>(c, sw, g, st, ws.perm, ws.glist, ws.gp, pruning, n_graphs);
+        if (e != cudaSuccess) return cuda_err(h, e, "local-moving launch");
+        if (sw.whole) break;
+        if (gc) batch_finish<M>(c, ws.ctrl, gc, n_graphs);
+        else move_finish<M>(c, ws.ctrl);
+      }
+    }
+    const Ctrl* hc = read_ctrl(h, c, &s, "local move");
+    if (!hc) return s;
+    if (hc->error & kErrTimeout)
+      return set_err(h, LOUVAIN_ERR_TIMEOUT, "a bounded grid-barrier wait of the local-moving phase ran out");
+    if (hc->error) return set_err(h, LOUVAIN_ERR_CUDA, "internal: hash table overflow in the local-moving phase");
+    if (hc->done || enq >= p.max_iterations) {
+      *li = hc->iterations;
+      *moves = (int64_t)hc->moves_pass;
+      return LOUVAIN_OK;
+    }
+  }
 }
 
 // One local-moving phase (Algorithm 2) on g from the state in ws (K, Sig, Cp, flags set).
@@ -925,6 +1034,8 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   cudaGraphExec_t g_first = nullptr, g_rest = nullptr;
   int64_t l_first = 0, l_rest = 0;
   const bool graphs = !h->prof.on && h->use_graphs;
+  if (det && graphs)
+    return sweep_phase<M>(h, c, g, st, first, glist, p, gc, n_graphs, li, moves, ms_graph, graphs_new);
   int32_t n_new = 0;
   double host_ms = 0.0;
   auto now = [] { return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count(); };

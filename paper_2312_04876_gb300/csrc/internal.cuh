@@ -44,10 +44,12 @@ struct GraphView {
 // serves every pass over the same arrays (the kernels read their vertex ranges here):
 //   [2b], [2b + 1]   start and count of degree bucket b < kNumBuckets - 1 in the perm list;
 //   [kStepGiant]     offset of the class-ordered giant list, then the giant range k0, k1 (plan indices);
-//   [kStepApply]     start and count of the deterministic Sigma apply.
+//   [kStepApply]     start and count of the deterministic Sigma apply;
+//   [kStepWide]      (sweep.cu) how the step applies its moves.
 constexpr int kStepWords = 20;
 constexpr int kStepGiant = 12;
 constexpr int kStepApply = 16;
+constexpr int kStepWide = 18;    // sweep: 1 if a block may make more moves in the step than it can keep
 
 // ---------------------------------------------------------------- prims.cu
 // Exclusive scan of in[0, n) into out[0, n) and out[n] = total; tile_tmp needs
@@ -253,6 +255,23 @@ template <class W>
 void compact_bucketed(Ctx& c, const int32_t* cperm, const int64_t* cb, const int64_t* hbeg, const int64_t* hend,
                       const int64_t* doff, const int32_t* itg, const W* iw, int32_t* otg, W* ow, const GiantPlan& gp,
                       Ctrl* ctrl);
+
+// ---------------------------------------------------------------- sweep.cu
+// Colour-class steps in one persistent launch: a whole local-moving phase, or the steps that one
+// iteration runs after its wide classes (then the caller finishes the iteration).
+struct SweepPlan {
+  void* sig2;                 // [n] second Sigma copy (a_t)
+  unsigned long long* state;  // [kSweepStateWords]
+  const int64_t* recs;        // device step records
+  int nsteps;
+  bool whole;
+  int scope;                  // Scope (persist.cuh)
+};
+constexpr int kSweepStateWords = 16;
+constexpr int kSweepMoves = 1024;  // moves of a narrow step that a block keeps
+template <class M>
+cudaError_t move_sweep(Ctx& c, const SweepPlan& sw, const GraphView<typename M::w_t>& g, const PassState<M>& st,
+                       const int32_t* perm, const int32_t* glist, const GiantPlan& gp, bool pruning, int32_t n_graphs);
 
 // ---------------------------------------------------------------- modularity.cu
 // Same value by degree-bucketed groups (dperm / hb: a degree-bucket sort of g), giant rows chunked.

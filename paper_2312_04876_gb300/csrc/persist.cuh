@@ -18,7 +18,8 @@ enum Scope { kCta = 0, kCluster = 1, kGrid = 2 };
 
 constexpr int kPersistThreads = 1024;
 constexpr int kClusterBlocks = 8;  // the portable maximum
-constexpr long long kBarrierPolls = 1LL << 19;  // built-in bound: x ~0.6 us a poll, about 0.3 s
+constexpr long long kBarrierPolls = 1LL << 23;  // built-in bound: x ~0.6 us a poll, about 5 s (a wide step
+                                                // of a graph of billions of arcs takes a good part of one)
 
 // Barrier word of one step: arrivals in the high bits, below them a sum the blocks publish with
 // their arrival, so that what every block must know about the step (how much work it left) comes

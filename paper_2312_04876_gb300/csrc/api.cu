@@ -297,7 +297,7 @@ louvain_status ensure_workspace(louvain_handle h, int64_t n, int64_t a) {
   ok = ok && dalloc(h, d, &ws.glist, gcap);
   ok = ok && dalloc(h, d, &ws.newid, n1 + 1) && dalloc(h, d, &ws.coff, n1 + 1) && dalloc(h, d, &ws.cdeg, n1 + 1) &&
        dalloc(h, d, &ws.len, n1 + 1) &&
-       dalloc(h, d, &ws.tile_tmp, scan_tmp_elems((int64_t)kNumBuckets * n1 + 8) + 8);  // class sort scans 5 n keys
+       dalloc(h, d, &ws.tile_tmp, scan_tmp_elems((int64_t)kDetBuckets * n1 + 8) + 8);  // class sort: keys per colour
   for (int r = 0; r < 2 && ok; r++)
     ok = dalloc(h, d, &ws.rows[r].hoff, n1 + 1) && dalloc(h, d, &ws.rows[r].hend, n1) &&
          dalloc(h, d, &ws.rows[r].doff, n1 + 1);
@@ -554,7 +554,7 @@ louvain_status degree_buckets(louvain_handle h, Ctx& c, const GraphView<W>& g, i
 struct ClassStep {
   int64_t start[kNumBuckets] = {};
   int64_t count[kNumBuckets] = {};
-  int64_t g0 = 0, g1 = 0;
+  int64_t g0 = 0, gm = 0, g1 = 0;  // giants; [g0, gm) of at most kSweepLongest arcs (deterministic)
   int64_t apply_start = 0, apply_count = 0;
 };
 
@@ -658,13 +658,75 @@ std::vector<int64_t> iteration_key(louvain_handle h, const Ctx& c, const GraphVi
   return k;
 }
 
-// Which steps a block could make more moves in than it keeps (sweep.cu): rows are dealt to `blocks`
-// blocks, a bucket's by groups of 4, 8, 32, 128, 512 and 1024 threads.
-bool step_is_wide(const ClassStep& cs, int64_t blocks) {
-  static const int64_t kGroups[kNumBuckets - 1] = {256, 128, 32, 8, 2, 1};
-  int64_t most = cs.g1 - cs.g0;
-  for (int b = 0; b < kNumBuckets - 1; b++) most += (cs.count[b] + blocks * kGroups[b] - 1) / (blocks * kGroups[b]) * kGroups[b];
-  return most > kSweepMoves;
+// Rows that a block takes at once, by kind: long giants, then degree buckets 5 to 0 (sweep.cu).
+constexpr int64_t kHubRows[7] = {1, 1, 2, 8, 16, 64, 128}, kLowRows[7] = {1, 1, 1, 8, 32, 128, 256};
+int64_t rows_of_kind(const ClassStep& cs, int x) { return x ? cs.count[6 - x] : cs.gm - cs.g0; }
+
+// Time of one block's batch of such rows, about (thousands of cycles), and of a pool giant's arcs on a
+// block (a giant of ~16,000 arcs spread over 16).
+constexpr int64_t kBatchCost[8] = {14, 10, 8, 7, 6, 5, 4, 6};
+constexpr int64_t kPoolBlocks = 16;
+
+// The record word that gives every block one kind of row (byte x: where kind x's blocks end, the pool
+// giants on the blocks that are left; bit 63 set), so that the kinds finish together: the smallest T
+// for which every kind's batches fit its share of the blocks in time T.  0 with one block, or more
+// than a byte counts, or where no row is long and the rows are many (planted partition of 100,003
+// vertices, 7,000 rows a step: 0.9 ms a phase by kinds, 0.7 without).  *wide: a block could make more
+// moves than it keeps.
+int64_t step_roles(const ClassStep& cs, int64_t blocks, bool hubs, bool* wide) {
+  const int64_t* const per = hubs ? kHubRows : kLowRows;
+  int64_t batches[8];
+  for (int x = 0; x < 7; x++) batches[x] = (rows_of_kind(cs, x) + per[x] - 1) / per[x];
+  batches[7] = (cs.g1 - cs.gm) * kPoolBlocks;
+  int64_t total = 0, most = 0, need[8];
+  for (int x = 0; x < 8; x++) total += batches[x] * kBatchCost[x];
+  for (int x = 0; x < 7; x++) most += (batches[x] + blocks - 1) / blocks * per[x];
+  *wide = most + cs.g1 - cs.gm > kSweepMoves;
+  if (blocks < 8 || blocks > 255) return 0;
+  if (!hubs) {  // many short rows balance by themselves, every kind on every block; few get a group each
+    int64_t sum = 0;
+    for (int x = 0; x < 7; x++) sum += batches[x];
+    if (sum > blocks) return 0;
+  }
+  auto fits = [&](int64_t T) {
+    int64_t sum = 0;
+    for (int x = 0; x < 8; x++) {
+      const int64_t rounds = std::max<int64_t>(1, T / kBatchCost[x]);  // batches a block takes within T
+      need[x] = (batches[x] + rounds - 1) / rounds;
+      sum += need[x];
+    }
+    return sum <= blocks;
+  };
+  int64_t lo = 0, hi = 15 + 8 * (total / blocks + 15);  // fits(hi): every kind within an eighth of the blocks
+  while (hi - lo > 1) {
+    const int64_t mid = (lo + hi) / 2;
+    if (fits(mid)) hi = mid;
+    else lo = mid;
+  }
+  if (!fits(hi)) return 0;
+  uint64_t w = 1ULL << 63;
+  int64_t end = 0, left = blocks;
+  for (int x = 0; x < 8; x++) left -= need[x];
+  if (batches[7] == 0)  // spare blocks to the kind with the most rounds
+    for (; left > 0; left--) {
+      int best = -1;
+      double worst = 0;
+      for (int x = 0; x < 7; x++)
+        if (need[x] > 0 && need[x] < batches[x] && (double)batches[x] * kBatchCost[x] / need[x] > worst) {
+          worst = (double)batches[x] * kBatchCost[x] / need[x];
+          best = x;
+        }
+      if (best < 0) break;
+      need[best]++;
+    }
+  most = 0;
+  for (int x = 0; x < 7; x++) {
+    if (need[x] > 0) most = std::max(most, (batches[x] + need[x] - 1) / need[x] * per[x]);
+    end += need[x];
+    w |= (uint64_t)end << (8 * x);
+  }
+  *wide = most + cs.g1 - cs.gm > kSweepMoves;
+  return (int64_t)w;
 }
 
 // Arcs of a step, about (a typical row length per bucket).
@@ -676,7 +738,8 @@ int64_t step_arcs(const ClassStep& cs) {
 }
 
 // Host image of the step records of `steps` (kStepWords each; the giant list offset from its base).
-void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64_t* out, int64_t blocks = 0) {
+void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64_t* out, int64_t blocks = 0,
+                        bool hubs = true) {
   for (size_t k = 0; k < steps.size(); k++) {
     int64_t* r = out + k * kStepWords;
     std::memset(r, 0, sizeof(int64_t) * kStepWords);
@@ -690,7 +753,12 @@ void write_step_records(const std::vector<ClassStep>& steps, int64_t goff, int64
     r[kStepGiant + 2] = cs.g1;
     r[kStepApply] = cs.apply_start;
     r[kStepApply + 1] = cs.apply_count;
-    r[kStepWide] = blocks > 0 && step_is_wide(cs, blocks) ? 1 : 0;
+    r[kStepLong] = cs.gm;
+    if (blocks > 0) {
+      bool wide = false;
+      r[kStepRoles] = step_roles(cs, blocks, hubs, &wide);
+      r[kStepWide] = wide ? 1 : 0;
+    }
   }
 }
 
@@ -802,41 +870,55 @@ louvain_status capture_iteration(louvain_handle h, Ctx& c0, const GraphView<type
 // Scope of the persistent class steps by the arcs of a step, about (step_arcs): one block up to 2048
 // (2,855 vertices, 1,122 arcs a step, 228 steps: 2.9 ms a phase on a block, 3.5 on a cluster; 5,486 arcs
 // a step: 8.5 against 5.2), a cluster up to 8000 (14,325 arcs a step: 1.0 ms on a cluster, 0.8 on the
-// grid), else the grid.  A class of over 8 million arcs keeps its per-bucket launches, as do those
-// before it: there a barrier more or less is nothing, and a launch's blocks retire as they finish
-// (24M-vertex grid, pass 1: 8.9 ms against 12.0 in the persistent launch).
-constexpr int64_t kSweepCtaArcs = 2048, kSweepClusterArcs = 8000, kSweepWideArcs = 8000000;
-// The deterministic phase's iterations: classes [0, f) as captured per-class launches, the others in
-// one persistent launch (sweep.cu); with f = 0 that launch runs the whole phase.
-template <class M>
-louvain_status sweep_phase(louvain_handle h, Ctx& c, const GraphView<typename M::w_t>& g, const PassState<M>& st,
-                           const std::vector<ClassStep>& steps, const int32_t* glist, const louvain_params& p,
-                           GraphCtl* gc, int32_t n_graphs, int32_t* li, int64_t* moves, float* ms_graph,
-                           int32_t* graphs_new) {
-  Workspace& ws = h->ws;
-  const bool pruning = p.pruning != 0;
-  louvain_status s;
-  size_t f = 0;
+// grid), else the grid.  A class with rows over 512 arcs keeps its per-bucket launches from 2 million
+// arcs on, as do the classes before it: there long rows' launches overlap (R-MAT 20: 52.9 ms a run,
+// 54.1 with a limit of 20 million).  Without such rows the persistent launch is the faster one
+// throughout (24M-vertex grid, 14 million arcs a class: 7.5 ms against 8.8 in pass 1; 512-graph batch
+// 57.0 against 60.9); the limit there only bounds how long a block may wait at a barrier.
+constexpr int64_t kSweepCtaArcs = 2048, kSweepClusterArcs = 8000, kSweepWideArcs = 2000000,
+                  kSweepWideLowArcs = 256000000;
+struct SweepLayout {
+  size_t f = 0;        // classes [0, f) keep their launches
+  Scope scope = kGrid;
+  int64_t blocks = 0;
+  bool hubs = false;   // a narrow class has a row of over 512 arcs
+};
+SweepLayout sweep_layout(const std::vector<ClassStep>& steps, int num_sms) {
+  SweepLayout l;
   int64_t arcs = 0, most = 0;
   for (size_t k = 0; k < steps.size(); k++) {
     const int64_t a = step_arcs(steps[k]);
-    if (a > kSweepWideArcs) {
-      f = k + 1;
+    const bool hubs = steps[k].count[4] + steps[k].count[5] > 0 || steps[k].g1 > steps[k].g0;
+    if (a > (hubs ? kSweepWideArcs : kSweepWideLowArcs)) {
+      l.f = k + 1;
       arcs = most = 0;
+      l.hubs = false;
     } else {
+      l.hubs |= hubs;
       arcs += a;
       most = std::max(most, a);
     }
   }
-  const int64_t narrow = (int64_t)(steps.size() - f), avg = narrow > 0 ? arcs / narrow : 0;
-  Scope scope = kGrid;
-  if (avg <= kSweepCtaArcs && most <= 16 * kSweepCtaArcs) scope = kCta;
-  else if (avg <= kSweepClusterArcs && most <= 16 * kSweepClusterArcs) scope = kCluster;
-  const int64_t blocks = scope == kCta ? 1 : (scope == kCluster ? kClusterBlocks : c.num_sms);
-  const int64_t words = (int64_t)steps.size() * kStepWords;
-  if ((s = ensure_desc(h, words)) != LOUVAIN_OK) return s;
-  write_step_records(steps, glist - ws.glist, h->dpin, blocks);
-  cudaMemcpyAsync(ws.desc, h->dpin, (size_t)words * sizeof(int64_t), cudaMemcpyHostToDevice, c.s);
+  const int64_t narrow = (int64_t)(steps.size() - l.f), avg = narrow > 0 ? arcs / narrow : 0;
+  if (avg <= kSweepCtaArcs && most <= 16 * kSweepCtaArcs) l.scope = kCta;
+  else if (avg <= kSweepClusterArcs && most <= 16 * kSweepClusterArcs) l.scope = kCluster;
+  l.blocks = l.scope == kCta ? 1 : (l.scope == kCluster ? kClusterBlocks : num_sms);
+  return l;
+}
+
+// The deterministic phase's iterations: classes [0, f) as captured per-class launches, the others in
+// one persistent launch (sweep.cu); with f = 0 that launch runs the whole phase.  The step records
+// are in ws.desc.
+template <class M>
+louvain_status sweep_phase(louvain_handle h, Ctx& c, const GraphView<typename M::w_t>& g, const PassState<M>& st,
+                           const std::vector<ClassStep>& steps, const SweepLayout& layout, const int32_t* glist,
+                           const louvain_params& p, GraphCtl* gc, int32_t n_graphs, int32_t* li, int64_t* moves,
+                           float* ms_graph, int32_t* graphs_new) {
+  Workspace& ws = h->ws;
+  const bool pruning = p.pruning != 0;
+  louvain_status s;
+  const size_t f = layout.f;
+  const int64_t narrow = (int64_t)(steps.size() - f);
   auto now = [] { return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count(); };
   const double t0 = now();
   cudaGraphExec_t exec = nullptr;
@@ -856,7 +938,7 @@ louvain_status sweep_phase(louvain_handle h, Ctx& c, const GraphView<typename M:
   }
   if (ms_graph) *ms_graph = (float)(now() - t0);
   if (graphs_new) *graphs_new = n_new;
-  const SweepPlan sw{ws.Sig2, ws.swstate, ws.desc + (int64_t)f * kStepWords, (int)narrow, f == 0, (int)scope};
+  const SweepPlan sw{ws.Sig2, ws.swstate, ws.desc + (int64_t)f * kStepWords, (int)narrow, f == 0, (int)layout.scope, layout.hubs};
   for (int32_t enq = 0;;) {
     // two iterations between host reads (one launch runs them all without wide classes)
     for (int k = 0; k < 2 && enq < p.max_iterations; k++, enq++) {
@@ -942,7 +1024,7 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
     if (ncol < 0) return colour_failure(h, c);
     if (colours) *colours = ncol;
     if (colour_rounds) *colour_rounds = (int32_t)rounds;
-    const int64_t nkeys = (int64_t)ncol * kNumBuckets;
+    const int64_t nkeys = (int64_t)ncol * kDetBuckets;
     if ((s = ensure_keys(h, nkeys)) != LOUVAIN_OK) return s;
     bucket_sort(c, KeyDesc{1, 1, 0, 0}, g.n, g.rbeg, g.rend, ws.colour, nullptr, nkeys, ws.perm, ws.keyoffs, ws.keycur, ws.tile_tmp,
                 nullptr);
@@ -972,20 +1054,14 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   const int32_t* glist = ws.glist;
   if (det) {
     for (int cl = 0; cl < ncol; cl++) {
-      const size_t base = (size_t)cl * kNumBuckets;
-      const int64_t cnt = ho[base + kNumBuckets] - ho[base + kNumBuckets - 1];
-      if (cnt > 0)
-        cudaMemcpyAsync(ws.glist + gofs[cl], ws.perm + ho[base + kNumBuckets - 1], (size_t)cnt * sizeof(int32_t),
-                        cudaMemcpyDeviceToDevice, c.s);
-      gofs[cl + 1] = gofs[cl] + (cnt > 0 ? cnt : 0);
+      const size_t base = (size_t)cl * kDetBuckets;
+      gofs[cl + 1] = gofs[cl] + ho[base + kDetBuckets] - ho[base + kNumBuckets - 1];
     }
   } else {
     const size_t gb = (size_t)(kNumBuckets - 1) * ncol;  // the giants of all classes, in class order
     glist = ws.perm + ho[gb];
     for (int cl = 0; cl <= ncol; cl++) gofs[cl] = ho[gb + cl] - ho[gb];
   }
-  if (giant_slots > 0 && (s = ensure_pool(h, c, giant_slots)) != LOUVAIN_OK) return s;
-  if (gofs[ncol] > 0) giant_move_plan<M>(c, g, glist, gofs[ncol], ws.gp, ws.ctrl);
   // the steps of an iteration: every class on its own; in fast mode the iterations after the first
   // may merge consecutive classes into groups (fewer, larger launches once most vertices are pruned)
   auto make_steps = [&](int group) {
@@ -995,8 +1071,8 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
       ClassStep cs;
       for (int b = 0; b < kNumBuckets - 1; b++) {
         if (det) {
-          cs.start[b] = ho[(size_t)c0 * kNumBuckets + b];
-          cs.count[b] = ho[(size_t)c0 * kNumBuckets + b + 1] - cs.start[b];
+          cs.start[b] = ho[(size_t)c0 * kDetBuckets + b];
+          cs.count[b] = ho[(size_t)c0 * kDetBuckets + b + 1] - cs.start[b];
         } else {
           cs.start[b] = ho[(size_t)b * ncol + c0];
           cs.count[b] = ho[(size_t)b * ncol + c1] - cs.start[b];
@@ -1005,8 +1081,10 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
       cs.g0 = gofs[c0];
       cs.g1 = gofs[c1];
       if (det) {
-        cs.apply_start = ho[(size_t)c0 * kNumBuckets];
-        cs.apply_count = ho[(size_t)c0 * kNumBuckets + kNumBuckets] - cs.apply_start;
+        const size_t base = (size_t)c0 * kDetBuckets;
+        cs.gm = cs.g0 + ho[base + kNumBuckets] - ho[base + kNumBuckets - 1];
+        cs.apply_start = ho[base];
+        cs.apply_count = ho[base + kDetBuckets] - cs.apply_start;
       }
       v.push_back(cs);
     }
@@ -1023,6 +1101,18 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   }
   const std::vector<ClassStep> first = make_steps(1);
   const std::vector<ClassStep> rest = later == ncol ? first : make_steps((ncol + later - 1) / later);
+  SweepLayout layout;
+  if (det) {
+    // the step records, from which the giants' list is gathered
+    layout = sweep_layout(first, c.num_sms);
+    const int64_t words = (int64_t)first.size() * kStepWords;
+    if ((s = ensure_desc(h, words)) != LOUVAIN_OK) return s;
+    write_step_records(first, 0, h->dpin, layout.blocks, layout.hubs);
+    cudaMemcpyAsync(ws.desc, h->dpin, (size_t)words * sizeof(int64_t), cudaMemcpyHostToDevice, c.s);
+    if (gofs[ncol] > 0) collect_giants(c, ws.desc, (int)first.size(), ws.perm, ws.glist);
+  }
+  if (giant_slots > 0 && (s = ensure_pool(h, c, giant_slots)) != LOUVAIN_OK) return s;
+  if (gofs[ncol] > 0) giant_move_plan<M>(c, g, glist, gofs[ncol], ws.gp, ws.ctrl);
   move_setup(c, ws.ctrl, tau, p.max_iterations);
   if (gc) batch_move_setup(c, gc, n_graphs, p.max_iterations);
   const bool pruning = p.pruning != 0;
@@ -1035,7 +1125,7 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   int64_t l_first = 0, l_rest = 0;
   const bool graphs = !h->prof.on && h->use_graphs;
   if (det && graphs)
-    return sweep_phase<M>(h, c, g, st, first, glist, p, gc, n_graphs, li, moves, ms_graph, graphs_new);
+    return sweep_phase<M>(h, c, g, st, first, layout, glist, p, gc, n_graphs, li, moves, ms_graph, graphs_new);
   int32_t n_new = 0;
   double host_ms = 0.0;
   auto now = [] { return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count(); };

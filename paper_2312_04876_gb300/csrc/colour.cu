@@ -54,6 +54,7 @@ enum { kJpCount = 0 /* 3 rotating list sizes */, kJpBar = 3 /* 3 barrier words *
        kJpRounds, kJpTrips, kJpWords };
 static_assert(kJpWords <= kJpStateWords, "state block");
 
+constexpr int kPersistThreads = 1024;
 // CH, the arcs of a list entry: 8 on low-degree graphs, else 32.
 constexpr int kJpQueue = 64;                          // queue slots of a warp (flushed from 32 on)
 // Entries a block keeps for itself, of rows of at most kJpKeep chunks.  With several blocks only a
@@ -447,9 +448,9 @@ __global__ void __launch_bounds__(kPersistThreads, 1) jp_persistent(JpArgs a, Pe
 
 template <int CH>
 static cudaError_t jp_launch(Scope sc, const Ctx& c, const JpArgs& a, const PersistBar& bar) {
-  if (sc == kCta) return scope_launch(sc, c, jp_persistent<kCta, CH>, kJpSmem, a, bar);
-  if (sc == kCluster) return scope_launch(sc, c, jp_persistent<kCluster, CH>, kJpSmem, a, bar);
-  return scope_launch(sc, c, jp_persistent<kGrid, CH>, kJpSmem, a, bar);
+  if (sc == kCta) return scope_launch(sc, c, jp_persistent<kCta, CH>, kPersistThreads, kJpSmem, a, bar);
+  if (sc == kCluster) return scope_launch(sc, c, jp_persistent<kCluster, CH>, kPersistThreads, kJpSmem, a, bar);
+  return scope_launch(sc, c, jp_persistent<kGrid, CH>, kPersistThreads, kJpSmem, a, bar);
 }
 
 int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g, const int32_t* perm, const int64_t* hb, uint64_t seed,

@@ -45,11 +45,16 @@ struct GraphView {
 //   [2b], [2b + 1]   start and count of degree bucket b < kNumBuckets - 1 in the perm list;
 //   [kStepGiant]     offset of the class-ordered giant list, then the giant range k0, k1 (plan indices);
 //   [kStepApply]     start and count of the deterministic Sigma apply;
-//   [kStepWide]      (sweep.cu) how the step applies its moves.
+//   [kStepLong], [kStepWide], [kStepRoles]  (sweep.cu) how the step is split and applied.
 constexpr int kStepWords = 20;
 constexpr int kStepGiant = 12;
 constexpr int kStepApply = 16;
+constexpr int kStepLong = 15;    // sweep: giants [k0, this) take a block each, [this, k1) the shared pool
 constexpr int kStepWide = 18;    // sweep: 1 if a block may make more moves in the step than it can keep
+constexpr int kStepRoles = 19;   // sweep: blocks by kind of row (0: every block takes every kind)
+// Degree buckets of the colour-class sort: the giants split at the longest row a block takes.
+constexpr int kDetBuckets = kNumBuckets + 1;
+constexpr int64_t kSweepLongest = 8192;
 
 // ---------------------------------------------------------------- prims.cu
 // Exclusive scan of in[0, n) into out[0, n) and out[n] = total; tile_tmp needs
@@ -61,7 +66,7 @@ void scan_exclusive_i32(Ctx& c, const int32_t* in, int64_t* out, int64_t n, int6
 void fill_i32(Ctx& c, int32_t* p, int32_t v, int64_t n);
 void iota_i32(Ctx& c, int32_t* p, int64_t n);
 
-// Sort key of bucket_sort: kind 0 degree bucket; 1 colour[i] * kNumBuckets + bucket; 2 degree bucket
+// Sort key of bucket_sort: kind 0 degree bucket; 1 colour[i] * kDetBuckets + bucket; 2 degree bucket
 // of deg64[i]; 3 (hash3(seed, pass, i) % classes) * kNumBuckets + bucket.
 struct KeyDesc {
   int kind = 0;
@@ -75,7 +80,7 @@ struct KeyDesc {
 };
 
 // Counting sort of vertex ids by key.  key_kind 0: degree bucket of (rend - rbeg); 1: colour *
-// kNumBuckets + degree bucket; 2: degree bucket of deg64[i].  Vertices with a negative key are
+// kDetBuckets + degree bucket (giants over kSweepLongest arcs in the last); 2: degree bucket of deg64[i].  Vertices with a negative key are
 // left out.  hist must hold nkeys + 1 int64; cursor nkeys int32.  Writes perm and offsets[nkeys+1]
 // (device).
 // max_deg (device, optional) receives the largest row length / deg64 value seen (atomicMax);
@@ -266,9 +271,12 @@ struct SweepPlan {
   int nsteps;
   bool whole;
   int scope;                  // Scope (persist.cuh)
+  bool hubs;                  // some row has over 512 arcs
 };
 constexpr int kSweepStateWords = 16;
 constexpr int kSweepMoves = 1024;  // moves of a narrow step that a block keeps
+// The class-ordered giant list of a phase from the step records' perm ranges.
+void collect_giants(Ctx& c, const int64_t* recs, int nsteps, const int32_t* perm, int32_t* glist);
 template <class M>
 cudaError_t move_sweep(Ctx& c, const SweepPlan& sw, const GraphView<typename M::w_t>& g, const PassState<M>& st,
                        const int32_t* perm, const int32_t* glist, const GiantPlan& gp, bool pruning, int32_t n_graphs);

@@ -16,7 +16,6 @@ namespace lv {
 
 enum Scope { kCta = 0, kCluster = 1, kGrid = 2 };
 
-constexpr int kPersistThreads = 1024;
 constexpr int kClusterBlocks = 8;  // the portable maximum
 constexpr long long kBarrierPolls = 1LL << 23;  // built-in bound: x ~0.6 us a poll, about 5 s (a wide step
                                                 // of a graph of billions of arcs takes a good part of one)
@@ -30,19 +29,23 @@ constexpr unsigned long long kBarSum = (1ULL << kBarShift) - 1;
 struct PersistBar {
   unsigned long long* word;  // [3] rotating words, zeroed before the launch
   long long max_spins;
-  unsigned long long epoch;  // barriers passed (each block's own copy)
+  unsigned epoch;            // barriers passed (each block's own copy)
 };
 
 // Every thread of every block calls it; thread 0 evaluates `value()` (below 2^52 in total) once the
-// whole block has arrived.  Writes before it are visible after it to all blocks of the scope.
-// *sum = the blocks' values.  Returns false (for the whole block) once a wait has run out; the block
-// then leaves.
-template <int SC, class V>
-__device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigned long long* sum, V value) {
+// whole block has arrived, and every thread runs `meanwhile()` between the arrival and the wait (loads
+// for the next step that no block of this one writes).  Writes before it are visible after it to all
+// blocks of the scope.  *sum = the blocks' values.  Returns false (for the whole block) once a wait has
+// run out; the block then leaves.  (The scope is a template argument: as a launch argument it cost a
+// one-block round 0.5 us.)
+template <int SC, class V, class W>
+__device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigned long long* sum, V value,
+                                              W meanwhile) {
   __shared__ unsigned long long sum_s;
   __syncthreads();
   if constexpr (SC == kCta) {
     if (threadIdx.x == 0) sum_s = value();
+    meanwhile();
     __syncthreads();
     *sum = sum_s;
     return true;
@@ -58,18 +61,24 @@ __device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigne
         if (blockIdx.x == 0) *(volatile unsigned long long*)clear = 0;
       }
       __syncwarp();
-      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      meanwhile();
+      __syncwarp();
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
       *sum = *(volatile unsigned long long*)w;
       return true;
     } else {
       __shared__ int ok_s;
+      unsigned long long x = 0;
       if (threadIdx.x == 0) {
-        int ok = 1;
         if (blockIdx.x == 0) *(volatile unsigned long long*)clear = 0;
         const unsigned long long add = (1ULL << kBarShift) + value();
-        unsigned long long x;
         asm volatile("atom.add.release.gpu.global.u64 %0, [%1], %2;" : "=l"(x) : "l"(w), "l"(add) : "memory");
         x += add;
+      }
+      meanwhile();
+      if (threadIdx.x == 0) {
+        int ok = 1;
         long long spins = 0;
         while ((x >> kBarShift) < gridDim.x) {
           if (++spins > b.max_spins) {
@@ -94,16 +103,21 @@ __device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigne
   }
 }
 
-// Launches kernel<SC>(args) with the scope's grid.  Returns the launch's status.
+template <int SC, class V>
+__device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigned long long* sum, V value) {
+  return scope_barrier<SC>(b, ctrl, sum, value, []() {});
+}
+
+// Launches kernel(args) with the scope's grid.  Returns the launch's status.
 template <class... P>
-inline cudaError_t scope_launch(Scope sc, const Ctx& c, void (*kernel)(P...), size_t smem, P... args) {
+inline cudaError_t scope_launch(Scope sc, const Ctx& c, void (*kernel)(P...), int threads, size_t smem, P... args) {
   if (smem > 48 * 1024) {  // the opt-in is idempotent and costs about a microsecond
     const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sc == kCta ? 1 : (sc == kCluster ? kClusterBlocks : c.num_sms));
-  cfg.blockDim = dim3(kPersistThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c.s;
   cudaLaunchAttribute at[1] = {};

@@ -145,7 +145,8 @@ __device__ __forceinline__ int sort_key(KeyDesc kd, int64_t i, const int64_t* rb
                            : hash3(kd.seed, (uint64_t)kd.pass, local_id(kd.seg, (int32_t)i));
     return b * kd.classes + (int)(h % (uint64_t)kd.classes);  // bucket-major: classes contiguous per bucket
   }
-  return colour[i] * kNumBuckets + b;
+  if (b == kNumBuckets - 1 && rend[i] - rbeg[i] > kSweepLongest) b = kDetBuckets - 1;
+  return colour[i] * kDetBuckets + b;
 }
 
 constexpr int kSmemKeys = 4096;

@@ -493,7 +493,7 @@ louvain_status validate_graph(louvain_handle h, Ctx& c, int64_t n, int64_t n_arc
   const Ctrl* hc = read_ctrl(h, c, &st, "validate offsets");
   if (!hc) return st;
   if (hc->cnt[0]) return set_err(h, LOUVAIN_ERR_INVALID, "offsets are not a monotone CSR offset array ending at n_arcs");
-  validate_arcs(c, n, offs, tg, w, fp, ctrl);
+  validate_arcs(c, n, n_arcs, offs, tg, w, fp, ctrl);
   hc = read_ctrl(h, c, &st, "validate arcs");
   if (!hc) return st;
   if (hc->cnt[1]) return set_err(h, LOUVAIN_ERR_INVALID, "arc target outside [0, n)");

@@ -347,7 +347,7 @@ void warm_init(Ctx& c, const PassState<M>& st, const int32_t* init, int64_t n);
 // ctrl->cnt[0..3] receive: bad offsets, bad targets, bad weights, asymmetry hash; ctrl->acc_f[0]
 // the weight total (double), ctrl->acc_i[0] the integer weight total (saturating).
 void validate_offsets(Ctx& c, int64_t n, int64_t n_arcs, const int64_t* offs, Ctrl* ctrl);
-void validate_arcs(Ctx& c, int64_t n, const int64_t* offs, const int32_t* tg, const void* w, bool fp, Ctrl* ctrl);
+void validate_arcs(Ctx& c, int64_t n, int64_t n_arcs, const int64_t* offs, const int32_t* tg, const void* w, bool fp, Ctrl* ctrl);
 // ctrl->cnt[5] += number of ids outside [0, hi).
 void validate_range(Ctx& c, const int32_t* ids, int64_t m, int64_t hi, Ctrl* ctrl);
 // zero ctrl->cnt[0..7], acc_i, acc_f

@@ -449,6 +449,17 @@ const int64_t* read_i64(louvain_handle h, Ctx& c, const int64_t* d, int64_t coun
   return *st == LOUVAIN_OK ? p : nullptr;
 }
 
+// Both at once: the control block (into *ctrl) and `count` int64.
+const int64_t* read_both(louvain_handle h, Ctx& c, const int64_t* d, int64_t count, const Ctrl** ctrl,
+                         louvain_status* st, const char* where) {
+  static_assert(sizeof(Ctrl) <= 1024, "the pinned buffer's first KiB");
+  *st = ensure_pinned(h, (size_t)count * sizeof(int64_t) + 8192);
+  if (*st != LOUVAIN_OK) return nullptr;
+  cudaMemcpyAsync(h->pin, h->ws.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c.s);
+  *ctrl = reinterpret_cast<const Ctrl*>(h->pin);
+  return read_i64(h, c, d, count, st, where);
+}
+
 const Ctrl* read_ctrl(louvain_handle h, Ctx& c, louvain_status* st, const char* where) {
   *st = ensure_pinned(h, 65536);
   if (*st != LOUVAIN_OK) return nullptr;
@@ -539,11 +550,10 @@ louvain_status degree_buckets(louvain_handle h, Ctx& c, const GraphView<W>& g, i
   cudaMemsetAsync(&ws.ctrl->gslots, 0, sizeof(unsigned long long), c.s);
   bucket_sort(c, KeyDesc{0, 1, 0, 0}, g.n, g.rbeg, g.rend, nullptr, nullptr, kNumBuckets, ws.dperm, ws.keyoffs,
               ws.keycur, ws.tile_tmp, nullptr, &ws.ctrl->gslots, g.n);
-  const int64_t* p = read_i64(h, c, ws.keyoffs, kNumBuckets + 1, &st, "degree buckets");
+  const Ctrl* hc = nullptr;
+  const int64_t* p = read_both(h, c, ws.keyoffs, kNumBuckets + 1, &hc, &st, "degree buckets");
   if (!p) return st;
   for (int b = 0; b <= kNumBuckets; b++) hb[b] = p[b];
-  const Ctrl* hc = read_ctrl(h, c, &st, "degree buckets");
-  if (!hc) return st;
   *giant_slots = (int64_t)hc->gslots;
   return LOUVAIN_OK;
 }
@@ -1214,12 +1224,11 @@ louvain_status aggregate_phase(louvain_handle h, Ctx& c, const GraphView<typenam
   cudaMemsetAsync(&ws.ctrl->gslots, 0, sizeof(unsigned long long), c.s);
   bucket_sort(c, KeyDesc{2, 1, 0, 0}, nc, nullptr, nullptr, nullptr, ws.cdeg, kNumBuckets, ws.cperm, ws.keyoffs,
               ws.keycur, ws.tile_tmp, nullptr, &ws.ctrl->gslots, nc);
-  const int64_t* q = read_i64(h, c, ws.keyoffs, kNumBuckets + 1, &s, "community buckets");
+  const Ctrl* hc = nullptr;
+  const int64_t* q = read_both(h, c, ws.keyoffs, kNumBuckets + 1, &hc, &s, "community buckets");
   if (!q) return s;
   int64_t cb[kNumBuckets + 1];
   for (int b = 0; b <= kNumBuckets; b++) cb[b] = cb_out[b] = q[b];
-  const Ctrl* hc = read_ctrl(h, c, &s, "community buckets");
-  if (!hc) return s;
   const int64_t giant_slots = (int64_t)hc->gslots;
   if (giant_slots > 0 && (s = ensure_pool(h, c, giant_slots)) != LOUVAIN_OK) return s;
   MergeArgs<M> a;
@@ -1375,13 +1384,12 @@ louvain_status run_impl(louvain_handle h, Ctx& c, int64_t n, int64_t n_arcs, con
     modularity_bucketed<M>(c, g0, C, reinterpret_cast<A*>(ws.tot), ws.ctrl, ws.dperm, hb0, ws.gpv);
     prof_end(h, c, kModularity, pm);
   }
-  const Ctrl* hc = read_ctrl(h, c, &s, "final modularity");
-  if (!hc) return s;
+  const Ctrl* hc = nullptr;
+  const int64_t* q = read_both(h, c, ws.newid + g.n, 1, &hc, &s, "final modularity");
+  if (!q) return s;
   if (hc->error) return set_err(h, LOUVAIN_ERR_CUDA, "internal: hash table overflow");
   prof_finish(h, *hc);
   out->q = hc->q;
-  const int64_t* q = read_i64(h, c, ws.newid + g.n, 1, &s, "final communities");
-  if (!q) return s;
   out->n_communities = q[0];
   if (stats) {
     for (int32_t lp = 0; lp < out->passes && lp < stats_cap; lp++) {
@@ -2228,11 +2236,10 @@ louvain_status louvain_aggregate(louvain_handle h, int64_t n, int64_t n_arcs, co
     scan_exclusive_i64(c, ws.len, d_out_offsets, n_comm, ws.tile_tmp);
     compact_bucketed<W>(c, ws.cperm, cb, rs.hoff, rs.hend, d_out_offsets, ws.tgA, reinterpret_cast<W*>(ws.wA),
                         d_out_targets, reinterpret_cast<W*>(d_out_weights), ws.gpv, ws.ctrl);
-    const int64_t* t = read_i64(h, c, d_out_offsets + n_comm, 1, &r, "aggregate total");
+    const Ctrl* cc = nullptr;
+    const int64_t* t = read_both(h, c, d_out_offsets + n_comm, 1, &cc, &r, "aggregate total");
     if (!t) return r;
     *out_arcs = t[0];
-    const Ctrl* cc = read_ctrl(h, c, &r, "aggregate end");
-    if (!cc) return r;
     if (cc->error) return set_err(h, LOUVAIN_ERR_CUDA, "internal: hash table overflow in aggregation");
     return LOUVAIN_OK;
   };

@@ -3,7 +3,7 @@
 // Some callers cannot call cudaMalloc: a host application whose memory manager owns all of the
 // device memory (a framework's caching allocator, or a fixed HBM budget already handed out), or a
 // latency-critical loop that cannot take the implicit device-wide synchronisation of
-// cudaMalloc / cudaFree.  For them this entry point runs the same three scan kernels as
+// cudaMalloc / cudaFree.  For them this entry point runs the same scan kernels as
 // louvain_exclusive_scan, but keeps the scratch (the per-tile sums) in a file-scope __device__
 // array instead of a handle's workspace.  Every GPU that loads the library holds that array
 // (128 KiB) until the process exits.

@@ -1,9 +1,11 @@
 // prims.cu -- exclusive scan, counting sort into degree / colour buckets, renumbering helpers.
 //
-// Scan (Algorithm 3's exclusiveScan, also used for renumbering in Algorithm 1): three launches,
-// tile sums -> scan of the tile sums in one block -> per-tile scan with the tile prefix.  Tiles of
-// 4096 elements; each warp of a tile owns 512 consecutive elements and scans them 32 at a time
-// with shuffles (coalesced loads and stores).  No inter-block waiting, so nothing can spin.
+// Scan (Algorithm 3's exclusiveScan, also used for renumbering in Algorithm 1).  Up to 32,768 elements
+// one block scans them in one launch: a small graph's run makes a dozen and a half scans, whose time is
+// launches (three of 3-5 us each before).  Beyond, tile sums and a per-tile scan whose block sums the
+// tiles before it, up to 2048 tiles (8.4M elements; their sums are 16 KB a block); beyond that a launch between them scans the tile
+// sums.  Tiles of 4096 elements; each warp of a tile owns 512 consecutive elements and scans them 32 at
+// a time with shuffles (coalesced loads and stores).  No inter-block waiting, so nothing can spin.
 #include "internal.cuh"
 
 namespace lv {
@@ -60,15 +62,29 @@ __global__ void __launch_bounds__(1024) scan_tile_prefix(long long* tsum, int64_
   if (threadIdx.x == 1023) *total = part[1023];
 }
 
-template <class T>
+// tsum holds the tiles' sums (kSums, the last block then also writes the total) or their exclusive scan.
+template <class T, bool kSums>
 __global__ void __launch_bounds__(kBlock) scan_tiles(const T* in, long long* out, int64_t n, const long long* tsum) {
-  __shared__ long long ws[kBlock / 32];
+  __shared__ long long ws[kBlock / 32], before[kBlock / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (kSums) {
+    long long b = 0;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += kBlock) b += tsum[t];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    if (lane == 0) before[warp] = b;
+  }
   int64_t base = (int64_t)blockIdx.x * kScanTile + warp * kScanWarpSpan;
   long long s = warp_chunk_sum(in, base, n);
   if (lane == 0) ws[warp] = s;
   __syncthreads();
-  long long run = tsum[blockIdx.x];
+  long long run = 0;
+  if (kSums) {
+    for (int w = 0; w < kBlock / 32; w++) run += before[w];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = run + tsum[blockIdx.x];
+  } else {
+    run = tsum[blockIdx.x];
+  }
   for (int w = 0; w < warp; w++) run += ws[w];
   for (int r = 0; r < kScanWarpSpan / 32; r++) {
     int64_t i = base + r * 32 + lane;
@@ -84,6 +100,48 @@ __global__ void __launch_bounds__(kBlock) scan_tiles(const T* in, long long* out
   }
 }
 
+// The whole scan by one block: four consecutive elements a thread and round.
+constexpr int64_t kScanBlockMax = 32768;
+template <class T>
+__global__ void __launch_bounds__(1024) scan_block(const T* in, long long* out, int64_t n) {
+  __shared__ long long ws[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long carry = 0;
+  for (int64_t base = 0; base < n; base += 4096) {
+    const int64_t i0 = base + 4 * (int64_t)threadIdx.x;
+    long long v[4], mine = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      v[k] = i0 + k < n ? (long long)in[i0 + k] : 0;
+      mine += v[k];
+    }
+    long long x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    long long w = ws[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    const long long below = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    long long run = carry + (warp > 0 ? below : 0) + x - mine;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (i0 + k < n) out[i0 + k] = run;
+      run += v[k];
+    }
+    carry += __shfl_sync(0xffffffffu, w, 31);
+    __syncthreads();  // ws is rewritten
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
 template <class T>
 static void scan_exclusive(Ctx& c, const T* in, int64_t* out, int64_t n, int64_t* tile_tmp) {
   long long* o = reinterpret_cast<long long*>(out);
@@ -92,10 +150,20 @@ static void scan_exclusive(Ctx& c, const T* in, int64_t* out, int64_t n, int64_t
     cudaMemsetAsync(out, 0, sizeof(int64_t), c.s);
     return;
   }
+  if (n <= kScanBlockMax) {
+    scan_block<T><<<1, 1024, 0, c.s>>>(in, o, n);
+    c.launches++;
+    return;
+  }
   int64_t tiles = (n + kScanTile - 1) / kScanTile;
   scan_tile_sums<T><<<(unsigned)tiles, kBlock, 0, c.s>>>(in, n, t);
+  if (tiles <= 2048) {
+    scan_tiles<T, true><<<(unsigned)tiles, kBlock, 0, c.s>>>(in, o, n, t);
+    c.launches += 2;
+    return;
+  }
   scan_tile_prefix<<<1, 1024, 0, c.s>>>(t, tiles, o + n);
-  scan_tiles<T><<<(unsigned)tiles, kBlock, 0, c.s>>>(in, o, n, t);
+  scan_tiles<T, false><<<(unsigned)tiles, kBlock, 0, c.s>>>(in, o, n, t);
   c.launches += 3;
 }
 
@@ -237,12 +305,86 @@ __global__ void __launch_bounds__(kBlock) k_key_scatter(KeyDesc kind, int64_t n,
   }
 }
 
+// The whole sort by one block, for few items and keys: counts, scan and places in shared memory.  A
+// small graph's sorts (two or three a pass) took eight launches each, 25-30 us; with the one-block scans
+// and one host read for the bucket bounds and the control block a run on 2,000 vertices went from 1.97
+// to 1.77 ms, on 10,000 from 3.24 to 3.03.  Beyond 8192 items a block's eight items a thread no longer
+// hide its latency and the histogram over many blocks is the faster one.
+constexpr int64_t kSortBlockMax = 8192;
+__global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const int64_t* rbeg, const int64_t* rend,
+                                                     const int32_t* colour, const int64_t* deg64, int nkeys,
+                                                     int32_t* perm, int64_t* offsets, unsigned long long* max_deg,
+                                                     unsigned long long* giant_slots, int64_t n_bound) {
+  __shared__ int32_t sh[kSmemKeys];
+  __shared__ int32_t ws[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int R = (int)kSortBlockMax / 1024;
+  int key[R];
+  for (int k = threadIdx.x; k < nkeys; k += 1024) sh[k] = 0;
+  __syncthreads();
+  unsigned long long gs = 0;
+  long long mx = 0;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int i = r * 1024 + threadIdx.x;
+    key[r] = -1;
+    if (i >= n) continue;
+    const long long dg = kind.kind == 2 ? deg64[i] : rend[i] - rbeg[i];
+    mx = dg > mx ? dg : mx;
+    if (giant_slots && bucket_of(dg, kind.giant_min) == kNumBuckets - 1)
+      gs += 1ULL << tbl_log2f(dg < n_bound ? dg : n_bound, kind.table_factor, 6, 31);
+    key[r] = sort_key(kind, i, rbeg, rend, colour, deg64);
+    if (key[r] >= 0) atomicAdd(&sh[key[r]], 1);
+  }
+  if (giant_slots && gs) atomicAdd(giant_slots, gs);
+  if (max_deg && mx > 0) atomicMax(max_deg, (unsigned long long)mx);
+  __syncthreads();
+  // exclusive scan of the counts, 1024 keys a round
+  int carry = 0;
+  for (int base = 0; base < nkeys; base += 1024) {
+    const int k = base + threadIdx.x;
+    const int v = k < nkeys ? sh[k] : 0;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    int w = ws[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    const int below = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    const int at = carry + (warp > 0 ? below : 0) + x - v;
+    if (k < nkeys) {
+      sh[k] = at;
+      offsets[k] = at;
+    }
+    carry += __shfl_sync(0xffffffffu, w, 31);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) offsets[nkeys] = carry;
+#pragma unroll
+  for (int r = 0; r < R; r++)
+    if (key[r] >= 0) perm[atomicAdd(&sh[key[r]], 1)] = r * 1024 + (int)threadIdx.x;
+}
+
 void bucket_sort(Ctx& c, KeyDesc key_kind, int64_t n, const int64_t* rbeg, const int64_t* rend, const int32_t* colour,
                  const int64_t* deg64, int64_t nkeys, int32_t* perm, int64_t* offsets, int32_t* cursor,
                  int64_t* tile_tmp, unsigned long long* max_deg, unsigned long long* giant_slots,
                  int64_t n_bound) {
   key_kind.giant_min = c.giant_min;
   key_kind.table_factor = c.table_factor;
+  if (n > 0 && n <= kSortBlockMax && nkeys <= kSmemKeys) {
+    k_sort_block<<<1, 1024, 0, c.s>>>(key_kind, (int)n, rbeg, rend, colour, deg64, (int)nkeys, perm, offsets, max_deg,
+                                      giant_slots, n_bound);
+    c.launches++;
+    return;
+  }
   cudaMemsetAsync(offsets, 0, (size_t)(nkeys + 1) * sizeof(int64_t), c.s);
   cudaMemsetAsync(cursor, 0, (size_t)nkeys * sizeof(int32_t), c.s);
   if (n <= 0) return;

@@ -107,8 +107,8 @@ typedef struct {
                                     those of the default placement (0) */
   int32_t table_factor;          /* hash-table slots per key a table may have to hold: 1, 2 or 4
                                     (tables up to full, half full or a quarter full; 0 = 2), for the
-                                    shared-memory tables of local moving and merging and the giant
-                                    rows' global tables.  Integer-weight results do not depend on it
+                                    shared-memory tables of merging, the giant rows' global tables
+                                    and, twice as many up to their capacity, those of local moving.  Integer-weight results do not depend on it
                                     (exact sums, ties by id); it trades probe length for memory */
   int32_t fast_sync_small;       /* fast mode on small graphs: 0 = where the input graph -- a batch:
                                     its mean graph -- fits in what the GPU holds in flight (1024

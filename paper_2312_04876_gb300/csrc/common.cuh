@@ -262,6 +262,35 @@ __device__ __forceinline__ void group_argmax(S& s, int32_t& c, S* ss, int32_t* s
   }
 }
 
+// Order-preserving 64-bit integer of a score, and back.
+__device__ __forceinline__ long long score_bits(long long s) { return s; }
+__device__ __forceinline__ long long score_bits(double s) {
+  const long long b = __double_as_longlong(s);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ void bits_score(long long b, long long& s) { s = b; }
+__device__ __forceinline__ void bits_score(long long b, double& s) {
+  s = __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffLL));
+}
+
+// Largest score of the warp, ties to the smallest community: three warp reductions (high word, low
+// word among its holders, community among theirs).
+template <class S>
+__device__ __forceinline__ void warp_best(S& s, int32_t& c) {
+  const long long b = score_bits(s);
+  const int32_t hi = (int32_t)(b >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = hi == mh ? (unsigned)b : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+  const unsigned id = hi == mh && lo == ml ? (unsigned)c : 0xffffffffu;
+  c = (int32_t)__reduce_min_sync(0xffffffffu, id);
+  bits_score(((long long)mh << 32) | ml, s);
+}
+__device__ __forceinline__ uint32_t warp_total(uint32_t x) { return __reduce_add_sync(0xffffffffu, x); }
+__device__ __forceinline__ float warp_total(float x) {
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
 // OR of a predicate over the group (uniform result; for a block it is also a barrier).
 template <int G>
 __device__ __forceinline__ bool group_any(bool p) {
@@ -307,23 +336,53 @@ __device__ __forceinline__ bool tbl_add(int32_t* keys, V* vals, unsigned size, i
   return false;
 }
 
-// tbl_add that also reports a new key: 0 = table full, 1 = added to an existing key, 2 = this call
-// claimed the key's slot (*slot = its index).
-template <class V>
-__device__ __forceinline__ int tbl_add_claim(int32_t* keys, V* vals, unsigned size, int shift, int32_t key, V w,
-                                             unsigned* slot) {
-  unsigned s = tbl_home(key, shift);
-  for (unsigned p = 0; p < size; p++) {
-    int32_t k = *((volatile int32_t*)&keys[s]);
-    if (k == key) { atomicAdd(&vals[s], w); return 1; }
-    if (k == kEmpty) {
-      int32_t old = atomicCAS(&keys[s], kEmpty, key);
-      if (old == kEmpty) { atomicAdd(&vals[s], w); *slot = s; return 2; }
-      if (old == key) { atomicAdd(&vals[s], w); return 1; }
-    }
-    s = (s + 1) & (size - 1);
+// Claims slot s for the key where `in` (predicated: under a branch each lane's and each key's swap would
+// wait for the one before); returns the slot's key before, the key itself where not `in`.
+__device__ __forceinline__ int32_t claim_if(bool in, int32_t* keys, unsigned s, int32_t key) {
+  int32_t old = key;
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\t@q atom.shared.cas.b32 %0, [%2], %3, %4;\n\t}"
+               : "+r"(old)
+               : "r"((int)in), "r"((unsigned)__cvta_generic_to_shared(keys + s)), "r"(kEmpty), "r"(key)
+               : "memory");
+  return old;
+}
+
+// Adds the U pairs (key[u], w[u]) where in[u] to a shared table of mask + 1 slots; s[u] = the key's slot.
+// One compare-and-swap a probe instead of a read, a compare and a swap, the U of them together; the
+// value is added once, after the probing.  Returns a bit per key whose slot this call claimed; *ok is
+// cleared if the table was full, which its size excludes.
+template <int U, class V>
+__device__ __forceinline__ unsigned tbl_put(const bool (&in)[U], int32_t* keys, V* vals, unsigned mask, int shift,
+                                            const int32_t (&key)[U], const V (&w)[U], unsigned (&s)[U], bool* ok) {
+  int32_t old[U];
+  bool left = false;
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    s[u] = tbl_home(key[u], shift);
+    old[u] = claim_if(in[u], keys, s[u], key[u]);
   }
-  return 0;
+#pragma unroll
+  for (int u = 0; u < U; u++) left |= old[u] != kEmpty && old[u] != key[u];
+  for (unsigned p = mask; left && p > 0; p--) {
+    left = false;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const bool again = old[u] != kEmpty && old[u] != key[u];
+      if (again) s[u] = (s[u] + 1) & mask;
+      const int32_t o = claim_if(again, keys, s[u], key[u]);
+      if (again) old[u] = o;
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) left |= old[u] != kEmpty && old[u] != key[u];
+  }
+  if (left) *ok = false;
+  unsigned own = 0;
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    if (in[u]) atomicAdd(&vals[s[u]], w[u]);
+    if (in[u] && old[u] == kEmpty) own |= 1u << u;
+  }
+  return own;
 }
 
 // Tables of {key, value} pairs (the giant-row pool): slot s is kv[2s] (key) and kv[2s + 1] (value

@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(kBlock) k_glm_insert(GraphView<typename M::w_t
                                                        const int64_t* krng, GiantAct ga) {
   typedef typename M::h_t H;
   constexpr int U = kLmChunk / kBlock;  // 2
-  __shared__ H red[32];
   if (*(volatile int32_t*)&ctrl->done) return;
   giant_range(krng, list, k0, k1);
   const int64_t q0 = p.chunk_off[k0], q1 = p.chunk_off[k1];
@@ -280,8 +279,9 @@ __global__ void __launch_bounds__(kBlock) k_glm_insert(GraphView<typename M::w_t
       if (cc[u] == d) kid += ww[u];
       else ok &= tbl_add_mark(kv, (unsigned)ts, 32 - lg, cc[u], ww[u], p.bits, off);
     }
-    kid = group_sum<kBlock>(kid, red);
-    if (threadIdx.x == 0 && kid != H(0)) atomicAdd(reinterpret_cast<H*>(p.kid) + k, kid);
+    __syncwarp();
+    kid = warp_total(kid);  // a sum over the block's warps costs three barriers a chunk
+    if ((threadIdx.x & 31) == 0 && kid != H(0)) atomicAdd(reinterpret_cast<H*>(p.kid) + k, kid);
   }
   if (!ok) atomicOr(&ctrl->error, kErrTableFull);
 }

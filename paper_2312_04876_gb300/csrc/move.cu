@@ -1,8 +1,8 @@
 // move.cu -- the local-moving phase of Algorithm 2 on the GPU.
 //
-// One group of G threads handles one vertex i (G by degree bucket: 4, 8, 32 lanes or a whole
-// block; rows above 4096 arcs take the multi-block path of giant.cu, whose tables live in global
-// memory).  The group streams i's arcs (scanCommunities with self = false), accumulates
+// One group of G threads handles one vertex i (G by degree bucket: 4, 8, 32 lanes or a block of
+// 128 or 512 threads; rows above 4096 arcs take the multi-block path of giant.cu, whose tables live in global
+// memory).  The group takes i's arcs (scanCommunities with self = false), accumulates
 // K_i->c for every neighbouring community c != C'[i] in an open-addressing table in shared
 // memory and K_i->d in registers, then scores
 // every candidate with the Eq. 2 numerator
@@ -71,319 +71,339 @@ __device__ __forceinline__ void flush_move_acc(Ctrl* ctrl, unsigned long long lo
   }
 }
 
-// Threads per block: warps with 1024-slot tables run in two-warp blocks, so a block (and its
-// shared memory) retires after two vertices instead of waiting for the slowest of eight.
-template <int G, int LOG>
-__host__ __device__ constexpr int lm_block() {
-  return (G == 32 && LOG >= 10) ? 64 : kBlock;
-}
+// Shape of a bucket's kernel: G threads a row, U arcs a thread, R rounds of them (G * U * R arcs hold the
+// bucket's longest row), tables of 2^LOG slots, blocks of T threads, B of them an SM (64 registers a
+// thread, 32 warps an SM).
+template <int G_, int U_, int R_, int LOG_, int T_, int B_>
+struct LmShape {
+  static constexpr int G = G_, U = U_, R = R_, LOG = LOG_, T = T_, B = B_, GPB = T_ / G_;
+  static constexpr bool kTable = G > 4;
+  template <class H>
+  static constexpr size_t smem() { return kTable ? (size_t)GPB * (1 << LOG) * (sizeof(int32_t) + sizeof(H)) : 0; }
+};
+typedef LmShape<4, 1, 1, 0, 256, 4> Lm0;
+typedef LmShape<8, 2, 1, 6, 256, 4> Lm1;
+typedef LmShape<32, 4, 1, 9, 128, 8> Lm2;
+typedef LmShape<128, 4, 1, 11, 128, 8> Lm3;
+typedef LmShape<512, 4, 1, 13, 512, 2> Lm4;
+typedef LmShape<512, 4, 2, 13, 512, 2> Lm5;
 
-// Blocks per SM the register budget is set for: two-warp blocks are held to 12 per SM by their
-// 16 KB of tables and lists anyway, so they may use up to 85 registers a thread.
-template <int G, int LOG>
-__host__ __device__ constexpr int lm_min_blocks() {
-  return lm_block<G, LOG>() == 64 ? 12 : (G <= 32 ? 4 : 3);
-}
-
-template <class M, int G, int LOG>
-__global__ void __launch_bounds__(lm_block<G, LOG>(), (lm_min_blocks<G, LOG>())) lm_kernel(LmArgs<M> a) {
+// One group per row.  Bound by the chain of dependent loads of a row and by how many rows an SM holds, so:
+// a row fits its group in one step (its targets stay in registers for the marks); the next row's head is
+// loaded during this one; the U swaps of a thread go out together; the thread that claims a slot loads
+// that community's Sigma at once and scores and clears the slot, without a list of claims; tables are a
+// quarter full where shared memory allows (half full, a 4096-arc row probes 2.5 times as long).
+// R-MAT 22 fast, ms of a run in rows of 129-512 arcs 4.88 -> 3.65, 513-2048 3.75 -> 3.43, 2049-4096
+// 3.49 -> 2.46, 17-128 3.23 -> 2.90, 5-16 1.27 -> 1.03, 1-4 0.94 -> 0.80, against a warp for up to 512 arcs
+// and 256 threads beyond, in rounds of four arcs a thread (the run 28.9 -> 23.8).  L1 and L2 then move
+// half of what they could and 37% of the issue slots are used: the rest is latency at 30 warps an SM.
+// Other shapes: 64 threads of eight arcs for 129-512 4.45, 256 of eight for 513-2048 3.71, 1024 of four
+// for 2049-4096 2.75 (and it holds the whole SM), 16 lanes of eight for 17-128 4.32, 24 warps of 85
+// registers even.
+template <class M, class P>
+__global__ void __launch_bounds__(P::T, P::B) lm_kernel(LmArgs<M> a) {
   typedef typename M::h_t H;
   typedef typename M::a_t A;
   typedef typename M::s_t S;
+  constexpr int G = P::G, U = P::U, R = P::R, LOG = P::LOG, T = P::T, GPB = P::GPB, NW = T / 32;
+  static_assert(G <= 32 || G == T, "a group is lanes of a warp or the block");
   Ctrl* ctrl = a.st.ctrl;
   if (*(volatile int32_t*)&ctrl->done) return;
-  constexpr int BS = lm_block<G, LOG>();
-  constexpr int GPB = G <= 32 ? BS / G : 1;
   // a captured iteration reads its list range from device memory (32-bit: counts and offsets are
   // below 2^31); the graph's arrays stay kernel parameters
-  int32_t lo = 0, hi = (int32_t)a.count;  // list[lo, hi)
+  unsigned lo = 0, hi = (unsigned)a.count;  // list[lo, hi)
   if (a.rng) {
-    lo = (int32_t)a.rng[0];
-    hi = lo + (int32_t)a.rng[1];
+    lo = (unsigned)a.rng[0];
+    hi = lo + (unsigned)a.rng[1];
   }
-  if (lo + (int)blockIdx.x * GPB >= hi) return;  // a fixed grid larger than this range
+  if (lo + blockIdx.x * GPB >= hi) return;  // a fixed grid larger than this range
   const GraphView<typename M::w_t>& g = a.g;
-  constexpr int SL = 1 << LOG;
-  constexpr int U = G >= 32 ? 4 : 2;  // arcs (and table slots) per lane per step
-  extern __shared__ __align__(16) unsigned char lm_dyn[];  // GPB tables of SL (key, value) slots
-  int32_t* skeys = reinterpret_cast<int32_t*>(lm_dyn);
-  H* svals = reinterpret_cast<H*>(lm_dyn + sizeof(int32_t) * GPB * SL);
-  // warp and block groups: the slots each vertex claimed, in claim order (a row has at most SL / 2
-  // distinct neighbouring communities, since tables hold at least twice the row's arcs), so the
-  // scoring visits and clears only occupied slots
-  constexpr bool kList = G >= 32;
-  constexpr int LMAX = kList ? SL / 2 : 1;
-  uint16_t* slist = reinterpret_cast<uint16_t*>(lm_dyn + (sizeof(int32_t) + sizeof(H)) * GPB * SL);
-  __shared__ int s_ncl;  // block groups: entries of the claimed-slot list
-  // per-warp reduction scratch, sized by the block's warps: static shared memory counts against
-  // the blocks an SM holds (13 instead of 11 two-warp blocks of 1024-slot tables)
-  constexpr int NW = BS / 32;
-  static_assert(BS % 32 == 0 && BS <= kBlock, "whole warps, at most kBlock threads");
+  extern __shared__ __align__(16) unsigned char lm_dyn[];  // GPB tables of 2^LOG (key, value) slots
+  const int gi = threadIdx.x / G, lane = threadIdx.x & (G - 1);
+  int32_t* const tk = reinterpret_cast<int32_t*>(lm_dyn) + (gi << LOG);
+  H* const tv = reinterpret_cast<H*>(lm_dyn + sizeof(int32_t) * (GPB << LOG)) + (gi << LOG);
   __shared__ S red_s[NW];
   __shared__ int32_t red_c[NW];
   __shared__ H red_h[NW];
-  __shared__ int32_t red_i[NW];
+  __shared__ int32_t red_i[1];
   __shared__ unsigned long long r_lo[NW], r_hi[NW], r_mv[NW];
   __shared__ double r_f[NW];
-
-  const int gib = G <= 32 ? (int)(threadIdx.x / G) : 0;
-  const unsigned lane = Grp<G>::lane();
-  for (int t = threadIdx.x; t < GPB * SL; t += BS) { skeys[t] = kEmpty; svals[t] = H(0); }
-  if (threadIdx.x == 0) s_ncl = 0;
-  __syncthreads();
-  int32_t* tk = skeys + gib * SL;  // this group's table
-  H* tv = svals + gib * SL;
-  uint16_t* cl = slist + gib * LMAX;  // this group's claimed-slot list
+  if constexpr (P::kTable) {
+    // 16 bytes a store; value 0 is 0u and 0.0f
+    for (int t = lane; t < (1 << LOG) / 4; t += G) {
+      reinterpret_cast<int4*>(tk)[t] = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
+      reinterpret_cast<int4*>(tv)[t] = make_int4(0, 0, 0, 0);
+    }
+    Grp<G>::sync();
+  }
   const A two_m_all = M::is_fp ? (A)ctrl->two_m_f : (A)ctrl->two_m_i;
   GraphCtl* const gcs = a.st.gc;
-  unsigned long long acc_lo = 0, acc_hi = 0, acc_mv = 0;
+  unsigned long long acc_lo = 0, acc_hi = 0, arcs = 0;
   double acc_f = 0.0;
-  unsigned long long ctr[6] = {0, 0, 0, 0, 0, 0};  // list, processed, arcs, candidates, moves, marks
+  unsigned listed = 0, processed = 0, cand = 0, moved = 0, marks = 0;
 
-  const int64_t ngroups = (int64_t)gridDim.x * GPB;
-  for (int32_t idx = lo + (int32_t)blockIdx.x * GPB + gib; idx < hi; idx += (int32_t)ngroups) {
-    const int32_t i = a.list[idx];
-    if (lane == 0) ctr[0]++;
-    // batched run: the graph of i, skipped once its local-moving phase has converged
-    GraphCtl* gcv = nullptr;
-    if (gcs) {
-      gcv = gcs + a.st.vg[i];
-      if (*(volatile int32_t*)&gcv->done) continue;
-    }
-    const A two_m = gcv ? (M::is_fp ? (A)gcv->two_m_f : (A)gcv->two_m_i) : two_m_all;
-    // row bounds, C'[i] and the flag are loaded together (the loads overlap)
-    const int64_t beg = g.rbeg[i], end = g.rend[i];
+  const unsigned stride = gridDim.x * GPB;
+  unsigned idx = lo + blockIdx.x * GPB + gi;
+  int32_t i1 = 0, i2 = 0, vg1 = 0;  // the next row, its head, and the one after it
+  int64_t b1 = 0, e1 = 0;
+  A k1 = A(0);
+  if (idx < hi) {
+    i1 = a.list[idx];
+    b1 = g.rbeg[i1];
+    e1 = g.rend[i1];
+    k1 = a.st.K[i1];
+    if (gcs) vg1 = a.st.vg[i1];
+    if (hi - idx > stride) i2 = a.list[idx + stride];
+  }
+  for (bool more = idx < hi; more;) {
+    const int32_t i = i1;
+    const int64_t beg = b1;
+    const int deg = (int)(e1 - b1);
+    const A ki = k1;
+    GraphCtl* const gcv = gcs ? gcs + vg1 : nullptr;  // batched run: the graph of i
     const int32_t d = a.st.Cp[i];
-    if (a.pruning) {
-      // every lane reads the flag and the group takes the OR, so the decision is uniform even if a
-      // neighbour re-marks i meanwhile; then i is marked as processed
-      const int f = a.st.flags[i];
-      if (!group_any<G>(f != 0)) continue;
-      if (lane == 0) a.st.flags[i] = 0;
+    // every thread reads the flag and the group takes the OR, so the decision is uniform even if a
+    // neighbour re-marks i meanwhile; then i is marked as processed
+    bool on = !a.pruning || a.st.flags[i] != 0;
+    A two_m = two_m_all;
+    if (gcv) {
+      on = on && !*(volatile int32_t*)&gcv->done;  // skipped once its local-moving phase has converged
+      two_m = M::is_fp ? (A)gcv->two_m_f : (A)gcv->two_m_i;
     }
-    const int64_t deg = end - beg;
-    if (lane == 0) { ctr[1]++; ctr[2] += (unsigned long long)deg; }
-    // K_i and Sigma_d are needed only for scoring; loaded here they overlap the arc loads (in the
-    // deterministic schedule Sigma does not change during a class; the fast schedule reads live values)
-    const A ki = a.st.K[i];
+    more = hi - idx > stride;
+    idx += stride;
+    if (more) {
+      i1 = i2;
+      b1 = g.rbeg[i1];
+      e1 = g.rend[i1];
+      k1 = a.st.K[i1];
+      if (gcs) vg1 = a.st.vg[i1];
+      if (hi - idx > stride) i2 = a.list[idx + stride];
+    }
+    if (lane == 0) listed++;
+    if (!group_any<G>(on)) continue;
+    if (lane == 0) {
+      if (a.pruning) a.st.flags[i] = 0;
+      processed++;
+      arcs += (unsigned long long)deg;
+    }
+    const int32_t* const rtg = g.tg + beg;
+    const typename M::w_t* const rw = g.w + beg;
+    int32_t jj[U], cc[U];
+    H ww[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int e = lane + u * G;
+      jj[u] = e < deg ? rtg[e] : i;
+      ww[u] = e < deg ? (H)rw[e] : H(0);
+    }
     const A sd = a.st.Sig[d];
-    const int lg = G > 32 ? tbl_log2f(deg, a.tf, 1, LOG) : tbl_log2f_fast(deg, a.tf, 1, LOG);
-    const unsigned size = 1u << lg;
-    const int shift = 32 - lg;
+    const int32_t lone = a.fast && lane == 0 ? a.st.csize[d] : 0;
+#pragma unroll
+    for (int u = 0; u < U; u++) cc[u] = a.st.Cp[jj[u]];
 
-    // scanCommunities(i, self = false): K_i->c into the table, K_i->d in registers.  U arcs per
-    // lane are loaded before their C'[j] gathers and the table updates, so each lane keeps U
-    // independent memory requests in flight.
     H kid = H(0);
-    bool ok = true;
-    unsigned ncl = 0;  // warp groups: entries of the claimed-slot list (uniform over the warp)
-    // every lane of a warp takes the same number of steps (the claim ballots need the whole warp)
-    // Warp and sub-warp groups index a row's arcs from its start in 32 bits (a row holds fewer than
-    // 2^31 arcs; fewer instructions per arc); the one-block kernels keep absolute 64-bit indices,
-    // which measured faster there.
-    typedef typename std::conditional<(G > 32), int64_t, int32_t>::type X;
-    const int32_t* const rtg = G > 32 ? g.tg : g.tg + beg;
-    const typename M::w_t* const rw = G > 32 ? g.w : g.w + beg;
-    const X rlo = G > 32 ? (X)beg : X(0), rhi = G > 32 ? (X)end : (X)deg;
-    for (X b0 = rlo; b0 < rhi; b0 += (X)(G * U)) {
-      const X e0 = b0 + (X)lane;
-      int32_t jj[U];
-      H ww[U];
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const X e = e0 + (X)(u * G);
-        jj[u] = e < rhi ? rtg[e] : i;
-        ww[u] = e < rhi ? (H)rw[e] : H(0);
-      }
-      int32_t cc[U];
-#pragma unroll
-      for (int u = 0; u < U; u++) cc[u] = jj[u] != i ? a.st.Cp[jj[u]] : kEmpty;
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const bool other = jj[u] != i && cc[u] != d;  // padding and i's self-loop are neither
-        if (jj[u] != i && cc[u] == d) kid += ww[u];
-        if constexpr (kList) {
-          // the new keys of this step are appended warp by warp to the claimed-slot list
-          int r = 1;
-          unsigned sl = 0;
-          if (other) r = tbl_add_claim(tk, tv, size, shift, cc[u], ww[u], &sl);
-          ok &= r != 0;
-          const unsigned b = __ballot_sync(0xffffffffu, r == 2);
-          if (b != 0u) {
-            unsigned base;
-            if constexpr (G == 32) {
-              base = ncl;
-              ncl += __popc(b);
-            } else {
-              unsigned t = 0;
-              if ((threadIdx.x & 31) == 0) t = (unsigned)atomicAdd(&s_ncl, __popc(b));
-              base = __shfl_sync(0xffffffffu, t, 0);
-            }
-            if (r == 2) cl[base + __popc(b & lanemask_lt())] = (uint16_t)sl;
-          }
-        } else if (other) {
-          ok &= tbl_add(tk, tv, size, shift, cc[u], ww[u]);
-        }
-      }
-    }
-    if (!ok) atomicOr(&ctrl->error, kErrTableFull);
-    Grp<G>::sync();
-    kid = group_sum<G>(kid, red_h);
-
-    // best community by the Eq. 2 numerator; the scan also clears the table.  The Sigma gathers of
-    // U slots per lane are issued together.
     S best = M::lowest();
     int32_t bc = 0x7fffffff;
-    // Warp and block groups score the slots listed at claim time (U per lane, their Sigma gathers
-    // issued together) and clear them, which leaves the table all-empty; sub-warp groups scan their
-    // small tables directly.
-    if constexpr (kList) {
-      const unsigned ncand = G == 32 ? ncl : (unsigned)*(volatile int*)&s_ncl;
-      for (unsigned k0 = lane; k0 < ncand; k0 += (unsigned)G * U) {
-        int32_t ck[U];
-        H vv[U];
-        A sg[U];
+    if constexpr (!P::kTable) {  // four arcs: the lanes compare their communities
+      const unsigned m = Grp<G>::mask();
+      const bool self = jj[0] == i;  // padding and i's self-loop
+      if (self) cc[0] = d;
+      H same = ww[0];
+      bool lower = false;
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-          const unsigned k = k0 + (unsigned)u * G;
-          ck[u] = kEmpty;
-          vv[u] = H(0);
-          if (k < ncand) {
-            const unsigned s = cl[k];
-            ck[u] = tk[s];
-            vv[u] = tv[s];
-            tk[s] = kEmpty;
-            tv[s] = H(0);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++) sg[u] = ck[u] != kEmpty ? a.st.Sig[ck[u]] : A(0);
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          if (ck[u] == kEmpty) continue;
-          ctr[3]++;
-          const S sc = M::score(vv[u], kid, ki, sg[u], sd, two_m);
-          if (better(sc, ck[u], best, bc)) { best = sc; bc = ck[u]; }
+      for (int o = 1; o < G; o++) {
+        const int32_t c2 = __shfl_xor_sync(m, cc[0], o);
+        const H w2 = __shfl_xor_sync(m, ww[0], o);
+        if (c2 == cc[0]) {
+          same += w2;
+          lower |= (lane ^ o) < lane;
         }
       }
+      const bool own = cc[0] != d && !lower;
+      const A sg = own ? a.st.Sig[cc[0]] : A(0);
+      kid = group_sum<G>(!self && cc[0] == d ? ww[0] : H(0), (H*)nullptr);
+      if (own) {
+        cand++;
+        best = M::score(same, kid, ki, sg, sd, two_m);
+        bc = cc[0];
+      }
+      group_argmax<G>(best, bc, (S*)nullptr, (int32_t*)nullptr);
     } else {
-      for (unsigned s0 = lane; s0 < size; s0 += (unsigned)G * U) {
-        int32_t ck[U];
-        H vv[U];
-        A sg[U];
+      const int lg = tbl_log2f_fast(deg, 2 * a.tf, 1, LOG);
+      const unsigned mask = (1u << lg) - 1;
+      unsigned claim[U];  // the slots this thread claimed: 16 bits a round
+      bool ok = true;
+#pragma unroll
+      for (int u = 0; u < U; u++) claim[u] = 0xffffffffu;
+#pragma unroll
+      for (int x = 0; x < R; x++) {
+        if (x > 0) {
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            const int e = lane + (x * U + u) * G;
+            jj[u] = e < deg ? rtg[e] : i;
+            ww[u] = e < deg ? (H)rw[e] : H(0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; u++) cc[u] = a.st.Cp[jj[u]];
+        }
+        unsigned s[U];
+        bool in[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-          const unsigned s = s0 + (unsigned)u * G;
-          ck[u] = s < size ? tk[s] : kEmpty;
-          vv[u] = H(0);
-          if (ck[u] != kEmpty) {
-            vv[u] = tv[s];
-            tk[s] = kEmpty;
-            tv[s] = H(0);
+          in[u] = jj[u] != i && cc[u] != d;
+          if (jj[u] != i && cc[u] == d) kid += ww[u];
+        }
+        const unsigned own = tbl_put<U>(in, tk, tv, mask, 32 - lg, cc, ww, s, &ok);
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if ((own >> u) & 1u) claim[u] = x ? ((claim[u] & 0xffffu) | (s[u] << 16)) : ((claim[u] & 0xffff0000u) | s[u]);
+      }
+      if (!ok) atomicOr(&ctrl->error, kErrTableFull);
+      A sg[U];
+      if constexpr (R == 1) {  // the claimed communities' totals are on their way during the wait
+#pragma unroll
+        for (int u = 0; u < U; u++) sg[u] = (claim[u] & 0xffffu) != 0xffffu ? a.st.Sig[cc[u]] : A(0);
+      }
+      if constexpr (G < 32) {
+        kid = group_sum<G>(kid, (H*)nullptr);
+      } else {
+        __syncwarp();
+        kid = warp_total(kid);
+      }
+      if (G > 32 && (threadIdx.x & 31) == 0) red_h[threadIdx.x >> 5] = kid;
+      Grp<G>::sync();  // every addition is made
+      if constexpr (G > 32) kid = warp_total((threadIdx.x & 31) < NW ? red_h[threadIdx.x & 31] : H(0));
+#pragma unroll
+      for (int x = 0; x < R; x++) {
+        int32_t key[U];
+        H val[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const unsigned sl = x ? claim[u] >> 16 : claim[u] & 0xffffu;
+          key[u] = kEmpty;
+          val[u] = H(0);
+          if (sl != 0xffffu) {
+            key[u] = R > 1 ? tk[sl] : cc[u];
+            val[u] = tv[sl];
+            tk[sl] = kEmpty;
+            tv[sl] = H(0);
           }
         }
+        if constexpr (R > 1) {
 #pragma unroll
-        for (int u = 0; u < U; u++) sg[u] = ck[u] != kEmpty ? a.st.Sig[ck[u]] : A(0);
+          for (int u = 0; u < U; u++) sg[u] = key[u] != kEmpty ? a.st.Sig[key[u]] : A(0);
+        }
 #pragma unroll
         for (int u = 0; u < U; u++) {
-          if (ck[u] == kEmpty) continue;
-          ctr[3]++;
-          const S sc = M::score(vv[u], kid, ki, sg[u], sd, two_m);
-          if (better(sc, ck[u], best, bc)) { best = sc; bc = ck[u]; }
+          if (key[u] == kEmpty) continue;
+          cand++;
+          const S sc = M::score(val[u], kid, ki, sg[u], sd, two_m);
+          if (better(sc, key[u], best, bc)) { best = sc; bc = key[u]; }
         }
+      }
+      if constexpr (G < 32) {
+        group_argmax<G>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+        Grp<G>::sync();  // the table is empty again
+      } else {
+        __syncwarp();  // for a warp's row: the table is empty again
+        warp_best(best, bc);
+      }
+      if constexpr (G > 32) {
+        if ((threadIdx.x & 31) == 0) {
+          red_s[threadIdx.x >> 5] = best;
+          red_c[threadIdx.x >> 5] = bc;
+        }
+        __syncthreads();
+        const bool in = (threadIdx.x & 31) < NW;
+        best = in ? red_s[threadIdx.x & 31] : M::lowest();
+        bc = in ? red_c[threadIdx.x & 31] : 0x7fffffff;
+        warp_best(best, bc);
       }
     }
-    group_argmax<G>(best, bc, red_s, red_c);
-    if (G > 32 && threadIdx.x == 0) s_ncl = 0;  // every thread read it before group_argmax's barriers
-    Grp<G>::sync();
 
     int mv = (bc != 0x7fffffff && best > S(0)) ? 1 : 0;
     if (mv && a.fast) {
       // singleton guard against lock-step swaps: a lone vertex joins another singleton
       // community only if that community's id is smaller
       int okm = 1;
-      if (lane == 0 && a.st.csize[d] == 1 && a.st.csize[bc] == 1 && bc > d) okm = 0;
-      mv = group_bcast<G>(okm, red_i);
-    }
-    if (mv) {
-      if (lane == 0) {
-        if (a.fast) {
-          atomic_add_a(&a.st.Sig[d], -ki);
-          atomic_add_a(&a.st.Sig[bc], ki);
-          atomicSub(&a.st.csize[d], 1);
-          atomicAdd(&a.st.csize[bc], 1);
-        } else {
-          a.st.mv_from[i] = d;
-          a.st.mv_to[i] = bc;
-        }
-        a.st.Cp[i] = bc;
-        if (gcv) {
-          if (M::is_fp) atomicAdd(&gcv->sum_f, (double)best);
-          else atomic_add_u128(&gcv->sum_lo, &gcv->sum_hi, (unsigned long long)best, 0ULL);
-        } else if (M::is_fp) {
-          acc_f += (double)best;
-        } else {
-          const unsigned long long b = (unsigned long long)best;
-          acc_lo += b;
-          if (acc_lo < b) acc_hi++;
-        }
-        acc_mv++;
-        ctr[4]++;
+      if (lane == 0 && lone == 1 && bc > d && a.st.csize[bc] == 1) okm = 0;
+      if constexpr (G > 32) {
+        if (lane == 0) red_i[0] = okm;
+        __syncthreads();
+        mv = red_i[0];
+      } else {
+        mv = __shfl_sync(Grp<G>::mask(), okm, 0, G);
       }
-      if (a.pruning)
-        for (X e0 = rlo + (X)lane; e0 < rhi; e0 += (X)(G * U)) {
-          int32_t jj[U];
+    }
+    if (!mv) continue;
+    if (lane == 0) {
+      if (a.fast) {
+        atomic_add_a(&a.st.Sig[d], -ki);
+        atomic_add_a(&a.st.Sig[bc], ki);
+        atomicSub(&a.st.csize[d], 1);
+        atomicAdd(&a.st.csize[bc], 1);
+      } else {
+        a.st.mv_from[i] = d;
+        a.st.mv_to[i] = bc;
+      }
+      a.st.Cp[i] = bc;
+      if (gcv) {
+        if (M::is_fp) atomicAdd(&gcv->sum_f, (double)best);
+        else atomic_add_u128(&gcv->sum_lo, &gcv->sum_hi, (unsigned long long)best, 0ULL);
+      } else if (M::is_fp) {
+        acc_f += (double)best;
+      } else {
+        const unsigned long long b = (unsigned long long)best;
+        acc_lo += b;
+        if (acc_lo < b) acc_hi++;
+      }
+      moved++;
+    }
+    if (a.pruning) {  // mark neighbours as unprocessed
 #pragma unroll
-          for (int u = 0; u < U; u++) {
-            const X e = e0 + (X)(u * G);
-            jj[u] = e < rhi ? rtg[e] : i;
-          }
+      for (int x = 0; x < R; x++)
 #pragma unroll
-          for (int u = 0; u < U; u++)
-            if (jj[u] != i) { a.st.flags[jj[u]] = 1; ctr[5]++; }  // mark neighbours as unprocessed
+        for (int u = 0; u < U; u++) {
+          const int e = lane + (x * U + u) * G;
+          const int32_t j = R == 1 ? jj[u] : (e < deg ? rtg[e] : i);
+          if (j != i) { a.st.flags[j] = 1; marks++; }
         }
     }
   }
-  flush_move_acc<M::is_fp>(ctrl, acc_lo, acc_hi, acc_mv, acc_f, r_lo, r_hi, r_mv, r_f);
+  flush_move_acc<M::is_fp>(ctrl, acc_lo, acc_hi, moved, acc_f, r_lo, r_hi, r_mv, r_f);
+  unsigned long long ctr[6] = {listed, processed, arcs, cand, moved, marks};
   block_add_counters<6, NW>(ctrl->lm_stat[a.bucket], ctr);
-}
-
-template <class M, int G, int LOG>
-static constexpr size_t lm_smem() {
-  return (size_t)(G <= 32 ? lm_block<G, LOG>() / G : 1) * (1 << LOG) *
-         (sizeof(int32_t) + sizeof(typename M::h_t) + (G >= 32 ? sizeof(uint16_t) / 2 : 0));
 }
 
 // Opts a kernel into more than 48 KB of dynamic shared memory, once per device (outside any graph
 // capture: move_prepare runs it for every instantiation before an iteration is captured).
-template <class M, int G, int LOG>
+template <class M, class P>
 static void lm_attr() {
-  constexpr size_t smem = lm_smem<M, G, LOG>();
+  constexpr size_t smem = P::template smem<typename M::h_t>();
   if (smem <= 48 * 1024) return;
   static std::atomic<unsigned long long> done{0};  // one bit per device
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && (done.load() >> dev) & 1ULL) return;
-  cudaFuncSetAttribute(lm_kernel<M, G, LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(lm_kernel<M, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (dev < 64) done.fetch_or(1ULL << dev);
 }
 
 void move_prepare() {
-  lm_attr<IntMode, 32, 10>();
-  lm_attr<IntMode, 256, 13>();
-  lm_attr<FpMode, 32, 10>();
-  lm_attr<FpMode, 256, 13>();
+  lm_attr<IntMode, Lm4>();
+  lm_attr<IntMode, Lm5>();
+  lm_attr<FpMode, Lm4>();
+  lm_attr<FpMode, Lm5>();
 }
 
-template <class M, int G, int LOG>
+template <class M, class P>
 static void launch_lm(Ctx& c, const LmArgs<M>& a, int max_blocks) {
-  constexpr int BS = lm_block<G, LOG>();
-  constexpr int GPB = G <= 32 ? BS / G : 1;
-  constexpr size_t smem = lm_smem<M, G, LOG>();
-  lm_attr<M, G, LOG>();
+  lm_attr<M, P>();
   // device-resident range: a.count is then an upper bound of the range (a power of two)
-  const int grid = grid_for(a.count, GPB, max_blocks * (kBlock / BS));
-  lm_kernel<M, G, LOG><<<grid, BS, smem, c.s>>>(a);
+  const int grid = grid_for(a.count, P::GPB, P::T < kBlock ? max_blocks * (kBlock / P::T) : max_blocks);
+  lm_kernel<M, P><<<grid, P::T, P::template smem<typename M::h_t>(), c.s>>>(a);
   c.launches++;
 }
 
@@ -401,12 +421,12 @@ void move_bucket(Ctx& c, int bucket, const GraphView<typename M::w_t>& g, const 
   a.tf = c.table_factor;
   const int cap = c.num_sms * c.lm_blocks_per_sm;
   switch (bucket) {
-    case 0: launch_lm<M, 4, 3>(c, a, cap); break;
-    case 1: launch_lm<M, 8, 5>(c, a, cap); break;
-    case 2: launch_lm<M, 32, 8>(c, a, cap); break;
-    case 3: launch_lm<M, 32, 10>(c, a, cap); break;
-    case 4: launch_lm<M, 256, 12>(c, a, cap); break;
-    case 5: launch_lm<M, 256, 13>(c, a, cap); break;
+    case 0: launch_lm<M, Lm0>(c, a, cap); break;
+    case 1: launch_lm<M, Lm1>(c, a, cap); break;
+    case 2: launch_lm<M, Lm2>(c, a, cap); break;
+    case 3: launch_lm<M, Lm3>(c, a, cap); break;
+    case 4: launch_lm<M, Lm4>(c, a, cap); break;
+    case 5: launch_lm<M, Lm5>(c, a, cap); break;
     default: break;  // giants go through giant_move
   }
 }

@@ -159,35 +159,6 @@ __device__ __forceinline__ typename M::s_t sweep_score(typename M::h_t kic, type
   else return (long long)(int32_t)two_m * (int32_t)(kic - kid) - (long long)(int32_t)ki * (int32_t)(sc - sd + ki);
 }
 
-// Order-preserving 64-bit integer of a score, and back.
-__device__ __forceinline__ long long score_bits(long long s) { return s; }
-__device__ __forceinline__ long long score_bits(double s) {
-  const long long b = __double_as_longlong(s);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
-}
-__device__ __forceinline__ void bits_score(long long b, long long& s) { s = b; }
-__device__ __forceinline__ void bits_score(long long b, double& s) {
-  s = __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffLL));
-}
-
-// Largest score of the warp, ties to the smallest community: three warp reductions (high word, low
-// word among its holders, community among theirs).
-template <class S>
-__device__ __forceinline__ void warp_best(S& s, int32_t& c) {
-  const long long b = score_bits(s);
-  const int32_t hi = (int32_t)(b >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
-  const unsigned lo = hi == mh ? (unsigned)b : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
-  const unsigned id = hi == mh && lo == ml ? (unsigned)c : 0xffffffffu;
-  c = (int32_t)__reduce_min_sync(0xffffffffu, id);
-  bits_score(((long long)mh << 32) | ml, s);
-}
-__device__ __forceinline__ uint32_t warp_total(uint32_t x) { return __reduce_add_sync(0xffffffffu, x); }
-__device__ __forceinline__ float warp_total(float x) {
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-
 // State of a step that its parts share.
 template <class M>
 struct Step {

@@ -33,8 +33,8 @@ __device__ __forceinline__ int64_t val_row(const int64_t* offs, int64_t lo, int6
 // A warp checks a contiguous range of arcs: one binary search finds its first row, then the ends of the
 // next 32 rows, one a lane, give every lane its arc's row by shuffles (a longer run of short or empty
 // rows falls back to the search).  By arcs and not by rows because rows are not alike: with 256 rows a
-// block, the blocks of R-MAT 20's hubs took 4.2 ms for arcs whose bytes take 0.04 (three single steps on
-// that graph with fp32 weights, two of them validating: 10.7 -> 3.5 ms).  What bounds it now is the
+// block, the blocks of R-MAT 20's hubs took 4.2 ms for arcs whose bytes take 0.04 (a modularity and an
+// aggregation on that graph with fp32 weights, both validating: 10.7 -> 3.5 ms).  What bounds it now is the
 // 64-bit hash of an arc.
 template <bool FP>
 __global__ void __launch_bounds__(kBlock) k_val_arcs(int64_t n, const int64_t* offs, const int32_t* tg, const void* wv,

@@ -102,7 +102,7 @@ struct SweepShared {
 };
 
 // A group of G threads: lanes of a warp, or whole warps that meet at a named barrier (64-thread groups
-// 1-8, 128-thread groups 1-4, 256-thread groups 9-10, the block 0).
+// 1-8, 128-thread groups 1-8, 256-thread groups 9-10, the block 0).
 template <int G, int T>
 __device__ __forceinline__ void team_sync() {
   if constexpr (G < 32) __syncwarp(Grp<G>::mask());
@@ -951,6 +951,10 @@ __global__ void __launch_bounds__(HUBS ? kSwThreads : kSwLowThreads, 1) lm_sweep
           if (head.on) load_arcs(a, head.i, head.beg, head.deg, tid & (G - 1), G, U, arcs);
         }
         sweep_rows<M, decltype(tag), T>(a, sh, sp, rl, first, cnt, step, head, arcs, roles == 0);
+        // Where one block takes every kind, the next kind's smaller groups write red_s and red_c: not
+        // before every warp of this group has read its last row's candidates there.
+        if constexpr (HUBS && G > 32)
+          if (!roles) team_sync<G, T>();
       };
       if constexpr (HUBS) {
         rows(Role<512, 8, 14, 2>(), 0, a.glist + rec[kStepGiant] + rec[kStepGiant + 1],

@@ -207,6 +207,12 @@ louvain_status louvain_workspace_bytes(louvain_handle h, size_t* bytes);
  * handle stays usable.  LOUVAIN_ERR_INVALID for k < 0. */
 louvain_status louvain_inject_alloc_failure(louvain_handle h, int32_t k);
 
+/* Fault injection for tests (the paper has no counterpart): on = 1 lets the handle's cluster and
+ * cooperative launches count as refused, as the driver refuses them where a context has only a part
+ * of the SMs; on = 0 ends that.  The deterministic mode then runs its colouring and class steps on
+ * one block, with the same results.  LOUVAIN_ERR_INVALID for another value. */
+louvain_status louvain_inject_launch_refusal(louvain_handle h, int32_t on);
+
 /* Message of the last failure on this handle ("" if none).  Valid until the next call. */
 const char* louvain_last_error(louvain_handle h);
 

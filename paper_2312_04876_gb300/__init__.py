@@ -227,6 +227,10 @@ class Louvain:
         """Make the k-th device allocation from now fail once (testing the out-of-memory path)."""
         self._check(self._lib.louvain_inject_alloc_failure(self._h, k))
 
+    def inject_launch_refusal(self, on: bool) -> None:
+        """Let cluster and cooperative launches count as refused (testing the one-block path)."""
+        self._check(self._lib.louvain_inject_launch_refusal(self._h, 1 if on else 0))
+
     def _check(self, st: int):
         if st != _native.OK:
             raise LouvainError(st, self._lib.louvain_last_error(self._h).decode())

@@ -156,6 +156,7 @@ struct louvain_handle_s {
   int64_t* dpin = nullptr;         // pinned staging of the step records
   int64_t dpin_cap = 0;
   uint64_t call_seq = 0;           // API calls so far (begin_call)
+  bool refuse_launch = false;      // cluster and cooperative launches count as refused (injected)
   int64_t fail_alloc_in = 0;       // > 0: the fail_alloc_in-th device allocation from now fails (injected)
   bool arcs_host = false;          // params.host_arcs of the current call: arc buffers in host memory
 };
@@ -1706,6 +1707,12 @@ louvain_status louvain_inject_alloc_failure(louvain_handle h, int32_t k) {
   return LOUVAIN_OK;
 }
 
+louvain_status louvain_inject_launch_refusal(louvain_handle h, int32_t on) {
+  if (!h || on < 0 || on > 1) return LOUVAIN_ERR_INVALID;
+  h->refuse_launch = on != 0;
+  return LOUVAIN_OK;
+}
+
 louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64_t* graph_vtx_offs, int64_t n_arcs,
                                  const int64_t* d_offsets, const int32_t* d_targets, const void* d_weights,
                                  louvain_wtype wtype, const louvain_params* p, void* stream, int32_t* d_membership,
@@ -1728,6 +1735,7 @@ louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -1822,6 +1830,7 @@ louvain_status run_entry(louvain_handle h, int64_t n, int64_t n_arcs, const int6
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -1924,6 +1933,7 @@ louvain_status louvain_update_graph(louvain_handle h, int64_t n_old, int64_t n_a
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   Workspace& ws = h->ws;
   if ((s = ensure_workspace(h, 1, 1)) != LOUVAIN_OK) return s;  // the control block
   const int64_t words = update_scratch_words(n_new, n_del) + scan_tmp_elems(n_new) + 8;
@@ -2083,6 +2093,7 @@ louvain_status louvain_modularity(louvain_handle h, int64_t n, int64_t n_arcs, c
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   const bool fp = wtype == LOUVAIN_W_FP32;
   if ((s = validate_graph(h, c, n, n_arcs, d_offsets, d_targets, d_weights, fp)) != LOUVAIN_OK) return s;
@@ -2119,6 +2130,7 @@ louvain_status louvain_colour(louvain_handle h, int64_t n, int64_t n_arcs, const
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   // the colour bitmaps and push chunks are sized from the arcs (ceil((deg + 1) / 32) words a vertex)
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   *n_colours = 0;
@@ -2158,6 +2170,7 @@ louvain_status louvain_local_move(louvain_handle h, int64_t n, int64_t n_arcs, c
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -2206,6 +2219,7 @@ louvain_status louvain_aggregate(louvain_handle h, int64_t n, int64_t n_arcs, co
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   const bool fp = wtype == LOUVAIN_W_FP32;
   if ((s = validate_graph(h, c, n, n_arcs, d_offsets, d_targets, d_weights, fp)) != LOUVAIN_OK) return s;
@@ -2303,6 +2317,7 @@ louvain_status louvain_exclusive_scan(louvain_handle h, const int64_t* d_in, int
   Ctx c;
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
+  c.one_block = h->refuse_launch;
   if ((s = ensure_workspace(h, count, 0)) != LOUVAIN_OK) return s;
   scan_exclusive_i64(c, d_in, d_out, count, h->ws.tile_tmp);
   if (total) {

@@ -108,9 +108,11 @@ __device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigne
   return scope_barrier<SC>(b, ctrl, sum, value, []() {});
 }
 
-// Launches kernel(args) with the scope's grid.  Returns the launch's status.
+// Launches kernel(args) with the scope's grid.  Returns the launch's status: a cluster or a cooperative
+// grid may be refused (a context that has only a part of the SMs); one block never is.
 template <class... P>
 inline cudaError_t scope_launch(Scope sc, const Ctx& c, void (*kernel)(P...), int threads, size_t smem, P... args) {
+  if (c.one_block && sc != kCta) return cudaErrorCooperativeLaunchTooLarge;
   if (smem > 48 * 1024) {  // the opt-in is idempotent and costs about a microsecond
     const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -59,7 +59,8 @@ struct SweepArgs {
   int whole;                  // 1: every iteration until the phase ends; 0: one iteration's steps
   int pruning;
   int n_graphs;
-  int all_wide;               // 1: the launch has fewer blocks than the records were made for
+  int all_wide;               // 1: the launch has fewer blocks than the records were made for: the blocks'
+                              // kinds of rows and move counts in them do not hold
   GiantPlan gp;
   unsigned long long* state;  // kSw* below, zeroed before the launch
 };
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(HUBS ? kSwThreads : kSwLowThreads, 1) lm_sweep
       load_descs(a, a.glist + r2[kStepGiant], r2[kStepLong], r2[kStepGiant + 2], sh.gd[(n + 2) % 3]);
     }
     const int64_t* r = sh.rec[(n + 1) & 3];
-    const unsigned long long roles = (unsigned long long)r[kStepRoles];
+    const unsigned long long roles = a.all_wide ? 0 : (unsigned long long)r[kStepRoles];
     head.i = -1;
     if (roles == 0) return;
     const int x = role_of(roles, blockIdx.x), b0 = x ? role_end(roles, x - 1) : 0;
@@ -897,7 +898,7 @@ __global__ void __launch_bounds__(HUBS ? kSwThreads : kSwLowThreads, 1) lm_sweep
       sp.wide = a.all_wide || rec[kStepWide] != 0;
       sp.nb = n & 1;
       sp.n_moves = &sh.n_moves[n % 3];
-      const unsigned long long roles = (unsigned long long)rec[kStepRoles];
+      const unsigned long long roles = a.all_wide ? 0 : (unsigned long long)rec[kStepRoles];
       // the last step's moves on the copy that lacks them
       {
         const SweepMove<M>* mv = sh.moves[(n + 1) & 1];

@@ -213,6 +213,12 @@ louvain_status louvain_inject_alloc_failure(louvain_handle h, int32_t k);
  * one block, with the same results.  LOUVAIN_ERR_INVALID for another value. */
 louvain_status louvain_inject_launch_refusal(louvain_handle h, int32_t on);
 
+/* Fault injection for tests (the paper has no counterpart): spins > 0 bounds the waits of the
+ * deterministic mode's class steps alone to that many polls, from a launch's `barrier`-th barrier on
+ * (0 = the first; louvain_params.wait_spins bounds every wait, and those of the colouring come
+ * first); spins = 0 ends that.  LOUVAIN_ERR_INVALID for a negative argument. */
+louvain_status louvain_inject_step_wait(louvain_handle h, int32_t spins, int32_t barrier);
+
 /* Message of the last failure on this handle ("" if none).  Valid until the next call. */
 const char* louvain_last_error(louvain_handle h);
 

@@ -231,6 +231,11 @@ class Louvain:
         """Let cluster and cooperative launches count as refused (testing the one-block path)."""
         self._check(self._lib.louvain_inject_launch_refusal(self._h, 1 if on else 0))
 
+    def inject_step_wait(self, spins: int, barrier: int = 0) -> None:
+        """Bound the class steps' waits alone to `spins` polls from a launch's `barrier`-th barrier on, 0
+        polls end that (testing a wait that runs out)."""
+        self._check(self._lib.louvain_inject_step_wait(self._h, spins, barrier))
+
     def _check(self, st: int):
         if st != _native.OK:
             raise LouvainError(st, self._lib.louvain_last_error(self._h).decode())

@@ -74,6 +74,7 @@ SIGNATURES = {
                                     _V, _V, _V, _I64, ctypes.POINTER(_I64)]),
     "louvain_inject_alloc_failure": (_I32, [_V, _I32]),
     "louvain_inject_launch_refusal": (_I32, [_V, _I32]),
+    "louvain_inject_step_wait": (_I32, [_V, _I32, _I32]),
     "louvain_run": (_I32, [_V, _I64, _I64, _V, _V, _V, _I32, ctypes.POINTER(Params), _V, _V, ctypes.POINTER(Result),
                            ctypes.POINTER(PassStats), _I32, ctypes.POINTER(_I32)]),
     "louvain_run_host": (_I32, [_V, _I64, _I64, _V, _V, _V, _I32, ctypes.POINTER(Params), _V, _V,

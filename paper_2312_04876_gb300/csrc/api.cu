@@ -66,6 +66,7 @@ struct Workspace {
   int64_t gt_slots_total = 0;
   unsigned* gt_bits = nullptr;
   int32_t* pool = nullptr;    // giant-row table pool: gt_slots_total {key, value} pairs
+  uint64_t pool_call = 0;     // the API call that took the pool and has not ended well, 0: none
   int32_t* dperm = nullptr;   // [n] vertex ids by degree bucket, kept for the whole pass
   DevAlloc desc_alloc;        // step records of captured iterations (kStepWords per class step)
   DevAlloc upd_alloc;         // batch graph update: deleted-pair set, row counters, scan scratch
@@ -156,6 +157,8 @@ struct louvain_handle_s {
   int64_t* dpin = nullptr;         // pinned staging of the step records
   int64_t dpin_cap = 0;
   uint64_t call_seq = 0;           // API calls so far (begin_call)
+  int32_t step_spins = 0;          // > 0: bound of the class steps' waits alone, from a launch's barrier
+  int32_t step_from = 0;           // step_from on (injected)
   bool refuse_launch = false;      // cluster and cooperative launches count as refused (injected)
   int64_t fail_alloc_in = 0;       // > 0: the fail_alloc_in-th device allocation from now fails (injected)
   bool arcs_host = false;          // params.host_arcs of the current call: arc buffers in host memory
@@ -333,9 +336,12 @@ louvain_status ensure_keys(louvain_handle h, int64_t nkeys) {
   return ensure_pinned(h, (size_t)(cap + 1) * sizeof(int64_t) + 4096);
 }
 
-// Shared pool of global-memory hash tables for the giant rows (all-empty between uses).
+// Shared pool of global-memory hash tables for the giant rows.  Every use leaves it empty, except one
+// that ends early (a bounded wait that ran out between a step's insertion and its scan): a call that
+// finds the pool taken by an earlier call that did not end well empties it first.
 louvain_status ensure_pool(louvain_handle h, Ctx& c, int64_t slots) {
   Workspace& ws = h->ws;
+  bool fresh = false;
   if (slots > ws.gt_slots_total) {
     free_all(ws.gt_alloc);
     ws.gt_slots_total = 0;
@@ -346,12 +352,16 @@ louvain_status ensure_pool(louvain_handle h, Ctx& c, int64_t slots) {
       free_all(ws.gt_alloc);
       return set_err(h, LOUVAIN_ERR_OOM, "giant hash-table pool allocation failed");
     }
-    pool_init(c, kv, total);
-    cudaMemsetAsync(bits, 0, (size_t)(total / 32) * 4, c.s);
     ws.pool = kv;
     ws.gt_bits = bits;
     ws.gt_slots_total = total;
+    fresh = true;
   }
+  if (fresh || (ws.pool_call != 0 && ws.pool_call != h->call_seq)) {
+    pool_init(c, ws.pool, ws.gt_slots_total);
+    cudaMemsetAsync(ws.gt_bits, 0, (size_t)(ws.gt_slots_total / 32) * 4, c.s);
+  }
+  ws.pool_call = h->call_seq;
   for (GiantPlan* gp : {&ws.gp, &ws.gpv}) {
     gp->slots = ws.pool;
     gp->bits = ws.gt_bits;
@@ -359,6 +369,9 @@ louvain_status ensure_pool(louvain_handle h, Ctx& c, int64_t slots) {
   }
   return LOUVAIN_OK;
 }
+
+// A call that used the pool has ended well.
+void pool_done(louvain_handle h) { h->ws.pool_call = 0; }
 
 // Device and pinned buffers for the step records of captured iterations (`words` int64).
 louvain_status ensure_desc(louvain_handle h, int64_t words) {
@@ -1713,6 +1726,13 @@ louvain_status louvain_inject_launch_refusal(louvain_handle h, int32_t on) {
   return LOUVAIN_OK;
 }
 
+louvain_status louvain_inject_step_wait(louvain_handle h, int32_t spins, int32_t barrier) {
+  if (!h || spins < 0 || barrier < 0) return LOUVAIN_ERR_INVALID;
+  h->step_from = barrier;
+  h->step_spins = spins;
+  return LOUVAIN_OK;
+}
+
 louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64_t* graph_vtx_offs, int64_t n_arcs,
                                  const int64_t* d_offsets, const int32_t* d_targets, const void* d_weights,
                                  louvain_wtype wtype, const louvain_params* p, void* stream, int32_t* d_membership,
@@ -1736,6 +1756,8 @@ louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -1786,6 +1808,7 @@ louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64
   cudaMemcpyAsync(stage, ws.gc, gbytes, cudaMemcpyDeviceToHost, c.s);
   cudaEventRecord(h->events[2], c.s);
   if ((s = sync(h, c, "batch end")) != LOUVAIN_OK) return s;
+  pool_done(h);
   const GraphCtl* gcs = reinterpret_cast<const GraphCtl*>(stage);
   int64_t ncomm = 0;
   int32_t max_pass = 0, iters = 0;
@@ -1831,6 +1854,8 @@ louvain_status run_entry(louvain_handle h, int64_t n, int64_t n_arcs, const int6
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -1884,6 +1909,7 @@ louvain_status run_entry(louvain_handle h, int64_t n, int64_t n_arcs, const int6
   if (!event_at(h, e_end)) return set_err(h, LOUVAIN_ERR_CUDA, "event creation failed");
   cudaEventRecord(h->events[e_end], c.s);
   if ((s = sync(h, c, "run end")) != LOUVAIN_OK) return s;
+  pool_done(h);
   if (res) {
     res->modularity = out.q;
     res->passes = out.passes;
@@ -1934,6 +1960,8 @@ louvain_status louvain_update_graph(louvain_handle h, int64_t n_old, int64_t n_a
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   Workspace& ws = h->ws;
   if ((s = ensure_workspace(h, 1, 1)) != LOUVAIN_OK) return s;  // the control block
   const int64_t words = update_scratch_words(n_new, n_del) + scan_tmp_elems(n_new) + 8;
@@ -2094,6 +2122,8 @@ louvain_status louvain_modularity(louvain_handle h, int64_t n, int64_t n_arcs, c
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   const bool fp = wtype == LOUVAIN_W_FP32;
   if ((s = validate_graph(h, c, n, n_arcs, d_offsets, d_targets, d_weights, fp)) != LOUVAIN_OK) return s;
@@ -2131,6 +2161,8 @@ louvain_status louvain_colour(louvain_handle h, int64_t n, int64_t n_arcs, const
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   // the colour bitmaps and push chunks are sized from the arcs (ceil((deg + 1) / 32) words a vertex)
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   *n_colours = 0;
@@ -2171,6 +2203,8 @@ louvain_status louvain_local_move(louvain_handle h, int64_t n, int64_t n_arcs, c
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if (p && p->giant_min_degree > 0) c.giant_min = p->giant_min_degree;
   if (p) c.wait_spins = p->wait_spins;
   if (p && p->table_factor > 0) c.table_factor = p->table_factor;
@@ -2200,7 +2234,8 @@ louvain_status louvain_local_move(louvain_handle h, int64_t n, int64_t n_arcs, c
     r = local_move_phase<M>(h, c, g, hb, gslots, *p, pass, tau, iterations, moves, 3);
     if (r != LOUVAIN_OK) return r;
     cudaMemcpyAsync(d_cprime, ws.Cp, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c.s);
-    return sync(h, c, "local move end");
+    if ((r = sync(h, c, "local move end")) == LOUVAIN_OK) pool_done(h);
+    return r;
   };
   return fp ? body(FpMode()) : body(IntMode());
 }
@@ -2220,6 +2255,8 @@ louvain_status louvain_aggregate(louvain_handle h, int64_t n, int64_t n_arcs, co
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if ((s = ensure_workspace(h, n, n_arcs)) != LOUVAIN_OK) return s;
   const bool fp = wtype == LOUVAIN_W_FP32;
   if ((s = validate_graph(h, c, n, n_arcs, d_offsets, d_targets, d_weights, fp)) != LOUVAIN_OK) return s;
@@ -2255,6 +2292,7 @@ louvain_status louvain_aggregate(louvain_handle h, int64_t n, int64_t n_arcs, co
     if (!t) return r;
     *out_arcs = t[0];
     if (cc->error) return set_err(h, LOUVAIN_ERR_CUDA, "internal: hash table overflow in aggregation");
+    pool_done(h);
     return LOUVAIN_OK;
   };
   return fp ? body(FpMode()) : body(IntMode());
@@ -2318,6 +2356,8 @@ louvain_status louvain_exclusive_scan(louvain_handle h, const int64_t* d_in, int
   c.s = reinterpret_cast<cudaStream_t>(stream);
   c.num_sms = h->num_sms;
   c.one_block = h->refuse_launch;
+  c.step_spins = h->step_spins;
+  c.step_from = (unsigned)h->step_from;
   if ((s = ensure_workspace(h, count, 0)) != LOUVAIN_OK) return s;
   scan_exclusive_i64(c, d_in, d_out, count, h->ws.tile_tmp);
   if (total) {

@@ -466,7 +466,7 @@ int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g, const int32_t* perm, cons
   const uint64_t gm = 0x9e3779b97f4a7c15ULL;
   a.key = mix64(mix64(seed + gm) + (uint64_t)pass + 2 * gm) + 3 * gm;
   for (int b = 0; b <= kNumBuckets; b++) a.hb[b] = (int32_t)hb[b];
-  PersistBar bar{jb.state + kJpBar, c.wait_spins > 0 ? c.wait_spins : kBarrierPolls, 0};
+  PersistBar bar{jb.state + kJpBar, c.wait_spins > 0 ? c.wait_spins : kBarrierPolls, 0, 0};
   // entries a round may hold at most with 8-arc chunks, and the arcs (typical row of each bucket)
   static const int64_t kChunks[kNumBuckets] = {1, 2, 16, 64, 256, 512, 0}, kArcs[kNumBuckets] = {3, 9, 48, 256, 1024, 3000, 12000};
   int64_t chunks = 0, arcs = 0;

@@ -30,6 +30,7 @@ struct PersistBar {
   unsigned long long* word;  // [3] rotating words, zeroed before the launch
   long long max_spins;
   unsigned epoch;            // barriers passed (each block's own copy)
+  unsigned from;             // the first barrier max_spins bounds; kBarrierPolls bounds those before (0 but in tests)
 };
 
 // Every thread of every block calls it; thread 0 evaluates `value()` (below 2^52 in total) once the
@@ -81,7 +82,7 @@ __device__ __forceinline__ bool scope_barrier(PersistBar& b, Ctrl* ctrl, unsigne
         int ok = 1;
         long long spins = 0;
         while ((x >> kBarShift) < gridDim.x) {
-          if (++spins > b.max_spins) {
+          if (++spins > b.max_spins && (b.epoch > b.from || spins > kBarrierPolls)) {
             atomicOr(&ctrl->error, kErrTimeout);
             ok = 0;
             break;

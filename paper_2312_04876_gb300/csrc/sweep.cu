@@ -1058,9 +1058,10 @@ cudaError_t move_sweep(Ctx& c, const SweepPlan& sw, const GraphView<typename M::
   a.state = sw.state;
   cudaError_t e = cudaMemsetAsync(sw.state, 0, kSwWords * sizeof(unsigned long long), c.s);
   if (e != cudaSuccess) return e;
-  const PersistBar bar{sw.state + kSwBar, c.wait_spins > 0 ? c.wait_spins : kBarrierPolls, 0};
+  const long long spins = c.step_spins > 0 ? c.step_spins : c.wait_spins;
+  const PersistBar bar{sw.state + kSwBar, spins > 0 ? spins : kBarrierPolls, 0, c.step_from};
   // a caller that bounds the waits gets the bounded barrier
-  const Scope sc = c.wait_spins > 0 ? kGrid : (Scope)sw.scope;
+  const Scope sc = spins > 0 ? kGrid : (Scope)sw.scope;
   e = sw.hubs ? sweep_launch<M, true>(sc, c, a, bar) : sweep_launch<M, false>(sc, c, a, bar);
   if (e != cudaSuccess && sc != kCta) {  // the scope cannot be launched here: one block can
     cudaGetLastError();

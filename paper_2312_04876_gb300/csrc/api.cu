@@ -42,7 +42,7 @@ struct Workspace {
   int32_t *perm = nullptr, *cperm = nullptr, *occ = nullptr, *counts = nullptr, *cursor = nullptr;
   int32_t *cverts = nullptr;
   int4* jrec = nullptr;       // colouring: vertex records, ready lists, colour bitmaps, state block
-  int4 *jl0 = nullptr, *jl1 = nullptr;
+  int4 *jl0 = nullptr, *jl1 = nullptr;  // (in memory that other parts of a pass use: ensure_workspace)
   int64_t jlist_cap = 0;
   unsigned* jused = nullptr;
   unsigned long long* jstate = nullptr;
@@ -280,9 +280,8 @@ louvain_status ensure_workspace(louvain_handle h, int64_t n, int64_t a) {
        dalloc(h, d, &ws.cperm, n1) && dalloc(h, d, &ws.occ, n1) && dalloc(h, d, &ws.counts, n1) &&
        dalloc(h, d, &ws.cursor, n1) && dalloc(h, d, &ws.cverts, n1);
   ws.jlist_cap = ac / 32 + n1 + 64;
-  ok = ok && dalloc(h, d, &ws.jrec, n1) && dalloc(h, d, &ws.jl0, ws.jlist_cap) && dalloc(h, d, &ws.jl1, ws.jlist_cap) &&
-       dalloc(h, d, &ws.jused, ac / 32 + n1 + 64) && dalloc(h, d, &ws.jstate, kJpStateWords) &&
-       dalloc(h, d, &ws.swstate, kSweepStateWords);
+  ok = ok && dalloc(h, d, &ws.jrec, n1) && dalloc(h, d, &ws.jused, ac / 32 + n1 + 64) &&
+       dalloc(h, d, &ws.jstate, kJpStateWords) && dalloc(h, d, &ws.swstate, kSweepStateWords);
   ok = ok && dalloc(h, d, &ws.flags, n1) && dalloc(h, d, &ws.dperm, n1) && dalloc(h, d, &ws.csz, n1);
   // giant plans: giant rows have > 4096 arcs, so there are at most A / 4097 of them; chunks of >= 512
   // arcs over their rows: <= gcap + A / 512; slices of >= 128 slots over tables of < 4 x the arcs:
@@ -291,17 +290,35 @@ louvain_status ensure_workspace(louvain_handle h, int64_t n, int64_t a) {
   for (GiantPlan* gp : {&ws.gp, &ws.gpv})
     ok = ok && dalloc(h, d, &gp->chunk_off, gcap + 1) && dalloc(h, d, &gp->tab_off, gcap + 1) &&
          dalloc(h, d, &gp->slice_off, gcap + 1) && dalloc(h, d, (int32_t**)&gp->kid, gcap) &&
-         dalloc(h, d, &gp->moved, gcap) && dalloc(h, d, &gp->active, gcap) &&
-         dalloc(h, d, (long long**)&gp->part_s, scap) &&
-         dalloc(h, d, &gp->part_c, scap) && dalloc(h, d, &gp->cowner, ccap) && dalloc(h, d, &gp->sowner, scap);
+         dalloc(h, d, &gp->moved, gcap) && dalloc(h, d, &gp->active, gcap) && dalloc(h, d, &gp->cowner, ccap);
   for (GiantPlan* gp : {&ws.gp, &ws.gpv}) {
     gp->chunk_cap = ccap;
     gp->slice_cap = scap;
   }
   ok = ok && dalloc(h, d, &ws.glist, gcap);
-  ok = ok && dalloc(h, d, &ws.newid, n1 + 1) && dalloc(h, d, &ws.coff, n1 + 1) && dalloc(h, d, &ws.cdeg, n1 + 1) &&
-       dalloc(h, d, &ws.len, n1 + 1) &&
-       dalloc(h, d, &ws.tile_tmp, scan_tmp_elems((int64_t)kDetBuckets * n1 + 8) + 8);  // class sort: keys per colour
+  // A pass colours its graph before it plans its giants, renumbers or aggregates, so each ready list lies
+  // where a plan's slices and two of those steps' per-vertex arrays do (16 bytes a vertex and half a
+  // byte an arc, either way): with lists of their own a run needed 32 bytes a vertex and a byte an arc more.
+  auto shared = [&](GiantPlan& gp, int64_t** a, int64_t** b, int4** list) {
+    int64_t at = 0;
+    auto part = [&](int64_t bytes) {
+      const int64_t p = at;
+      at += (bytes + 255) & ~(int64_t)255;
+      return p;
+    };
+    const int64_t s = part(scap * 8), c = part(scap * 4), o = part(scap * 4), x = part((n1 + 1) * 8), y = part((n1 + 1) * 8);
+    char* p = nullptr;
+    if (!dalloc(h, d, &p, std::max<int64_t>(at, ws.jlist_cap * (int64_t)sizeof(int4)))) return false;
+    gp.part_s = p + s;
+    gp.part_c = reinterpret_cast<int32_t*>(p + c);
+    gp.sowner = reinterpret_cast<int32_t*>(p + o);
+    *a = reinterpret_cast<int64_t*>(p + x);
+    *b = reinterpret_cast<int64_t*>(p + y);
+    *list = reinterpret_cast<int4*>(p);
+    return true;
+  };
+  ok = ok && shared(ws.gp, &ws.cdeg, &ws.len, &ws.jl0) && shared(ws.gpv, &ws.newid, &ws.coff, &ws.jl1);
+  ok = ok && dalloc(h, d, &ws.tile_tmp, scan_tmp_elems((int64_t)kDetBuckets * n1 + 8) + 8);  // class sort: keys per colour
   for (int r = 0; r < 2 && ok; r++)
     ok = dalloc(h, d, &ws.rows[r].hoff, n1 + 1) && dalloc(h, d, &ws.rows[r].hend, n1) &&
          dalloc(h, d, &ws.rows[r].doff, n1 + 1);

@@ -570,22 +570,26 @@ louvain_status colour_failure(louvain_handle h, Ctx& c) {
   return set_err(h, LOUVAIN_ERR_CUDA, "internal: " + what);
 }
 
-// Per-pass degree buckets of graph g into ws.dperm with host offsets hb[kNumBuckets + 1];
-// *giant_slots = table slots its giant vertices need.
+// The giant rows of a graph: table slots they need, arcs in all, the longest row's.
+struct GiantRows {
+  int64_t slots = 0, arcs = 0, longest = 0;
+};
+
+// Per-pass degree buckets of graph g into ws.dperm with host offsets hb[kNumBuckets + 1], and its giants.
 template <class W>
 louvain_status degree_buckets(louvain_handle h, Ctx& c, const GraphView<W>& g, int64_t hb[kNumBuckets + 1],
-                              int64_t* giant_slots) {
+                              GiantRows* giants) {
   Workspace& ws = h->ws;
   louvain_status st = ensure_keys(h, kNumBuckets);
   if (st != LOUVAIN_OK) return st;
-  cudaMemsetAsync(&ws.ctrl->gslots, 0, sizeof(unsigned long long), c.s);
+  cudaMemsetAsync(ws.ctrl->giants, 0, sizeof(ws.ctrl->giants), c.s);
   bucket_sort(c, KeyDesc{0, 1, 0, 0}, g.n, g.rbeg, g.rend, nullptr, nullptr, kNumBuckets, ws.dperm, ws.keyoffs,
-              ws.keycur, ws.tile_tmp, nullptr, &ws.ctrl->gslots, g.n);
+              ws.keycur, ws.tile_tmp, nullptr, ws.ctrl->giants, g.n);
   const Ctrl* hc = nullptr;
   const int64_t* p = read_both(h, c, ws.keyoffs, kNumBuckets + 1, &hc, &st, "degree buckets");
   if (!p) return st;
   for (int b = 0; b <= kNumBuckets; b++) hb[b] = p[b];
-  *giant_slots = (int64_t)hc->gslots;
+  *giants = GiantRows{(int64_t)hc->giants[0], (int64_t)hc->giants[1], (int64_t)hc->giants[2]};
   return LOUVAIN_OK;
 }
 
@@ -770,11 +774,10 @@ int64_t step_roles(const ClassStep& cs, int64_t blocks, bool hubs, bool* wide) {
   return (int64_t)w;
 }
 
-// Arcs of a step, about (a typical row length per bucket).
+// Arcs of a step, about.
 int64_t step_arcs(const ClassStep& cs) {
-  static const int64_t kArcs[kNumBuckets - 1] = {3, 9, 48, 256, 1024, 3000};
-  int64_t a = 12000 * (cs.g1 - cs.g0);
-  for (int b = 0; b < kNumBuckets - 1; b++) a += cs.count[b] * kArcs[b];
+  int64_t a = kTypicalArcs[kNumBuckets - 1] * (cs.g1 - cs.g0);
+  for (int b = 0; b < kNumBuckets - 1; b++) a += cs.count[b] * kTypicalArcs[b];
   return a;
 }
 
@@ -924,7 +927,7 @@ struct SweepLayout {
   int64_t blocks = 0;
   bool hubs = false;   // a narrow class has a row of over 512 arcs
 };
-SweepLayout sweep_layout(const std::vector<ClassStep>& steps, int num_sms) {
+SweepLayout sweep_layout(const std::vector<ClassStep>& steps, const GiantRows& giants, int num_sms) {
   SweepLayout l;
   int64_t arcs = 0, most = 0;
   for (size_t k = 0; k < steps.size(); k++) {
@@ -939,6 +942,11 @@ SweepLayout sweep_layout(const std::vector<ClassStep>& steps, int num_sms) {
       arcs += a;
       most = std::max(most, a);
     }
+  }
+  // the scope goes by the giants' own lengths where they are more
+  if (l.f < steps.size() && steps.back().g1 > steps[l.f].g0) {
+    arcs += std::max<int64_t>(0, giants.arcs - kTypicalArcs[kNumBuckets - 1] * steps.back().g1);
+    most = std::max(most, giants.longest);
   }
   const int64_t narrow = (int64_t)(steps.size() - l.f), avg = narrow > 0 ? arcs / narrow : 0;
   if (avg <= kSweepCtaArcs && most <= 16 * kSweepCtaArcs) l.scope = kCta;
@@ -1012,7 +1020,7 @@ louvain_status sweep_phase(louvain_handle h, Ctx& c, const GraphView<typename M:
 // Fills *li and *moves.  Deterministic mode colours g first.
 template <class M>
 louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typename M::w_t>& g, const int64_t hb[],
-                                int64_t giant_slots, const louvain_params& p, int32_t pass, double tau, int32_t* li,
+                                const GiantRows& giants, const louvain_params& p, int32_t pass, double tau, int32_t* li,
                                 int64_t* moves, size_t ev_colour_done, GraphCtl* gc = nullptr,
                                 const int32_t* vg = nullptr, int32_t n_graphs = 0, int32_t* colours = nullptr,
                                 int32_t* colour_rounds = nullptr, float* ms_graph = nullptr,
@@ -1059,7 +1067,7 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
     cudaError_t ce;
     const int pm = prof_begin(h, c);
     int64_t rounds = 0;
-    ncol = jp_colour(c, gs, ws.dperm, hb, p.seed, pass, ws.colour, jb, ws.ctrl, h->pin, &ce, seg, &rounds);
+    ncol = jp_colour(c, gs, ws.dperm, hb, p.seed, pass, ws.colour, jb, ws.ctrl, h->pin, &ce, giants.arcs, seg, &rounds);
     prof_end(h, c, kColour, pm);
     if (ce != cudaSuccess) return cuda_err(h, ce, "colouring");
     if (ncol < 0) return colour_failure(h, c);
@@ -1145,14 +1153,14 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   SweepLayout layout;
   if (det) {
     // the step records, from which the giants' list is gathered
-    layout = sweep_layout(first, c.num_sms);
+    layout = sweep_layout(first, giants, c.num_sms);
     const int64_t words = (int64_t)first.size() * kStepWords;
     if ((s = ensure_desc(h, words)) != LOUVAIN_OK) return s;
     write_step_records(first, 0, h->dpin, layout.blocks, layout.hubs);
     cudaMemcpyAsync(ws.desc, h->dpin, (size_t)words * sizeof(int64_t), cudaMemcpyHostToDevice, c.s);
     if (gofs[ncol] > 0) collect_giants(c, ws.desc, (int)first.size(), ws.perm, ws.glist);
   }
-  if (giant_slots > 0 && (s = ensure_pool(h, c, giant_slots)) != LOUVAIN_OK) return s;
+  if (giants.slots > 0 && (s = ensure_pool(h, c, giants.slots)) != LOUVAIN_OK) return s;
   if (gofs[ncol] > 0) giant_move_plan<M>(c, g, glist, gofs[ncol], ws.gp, ws.ctrl);
   move_setup(c, ws.ctrl, tau, p.max_iterations);
   if (gc) batch_move_setup(c, gc, n_graphs, p.max_iterations);
@@ -1252,15 +1260,15 @@ louvain_status aggregate_phase(louvain_handle h, Ctx& c, const GraphView<typenam
   cudaMemcpyAsync(rs.hend, rs.hoff, (size_t)nc * sizeof(int64_t), cudaMemcpyDeviceToDevice, c.s);
   // communities by total-degree bucket
   if ((s = ensure_keys(h, kNumBuckets)) != LOUVAIN_OK) return s;
-  cudaMemsetAsync(&ws.ctrl->gslots, 0, sizeof(unsigned long long), c.s);
+  cudaMemsetAsync(ws.ctrl->giants, 0, sizeof(ws.ctrl->giants), c.s);
   bucket_sort(c, KeyDesc{2, 1, 0, 0}, nc, nullptr, nullptr, nullptr, ws.cdeg, kNumBuckets, ws.cperm, ws.keyoffs,
-              ws.keycur, ws.tile_tmp, nullptr, &ws.ctrl->gslots, nc);
+              ws.keycur, ws.tile_tmp, nullptr, ws.ctrl->giants, nc);
   const Ctrl* hc = nullptr;
   const int64_t* q = read_both(h, c, ws.keyoffs, kNumBuckets + 1, &hc, &s, "community buckets");
   if (!q) return s;
   int64_t cb[kNumBuckets + 1];
   for (int b = 0; b <= kNumBuckets; b++) cb[b] = cb_out[b] = q[b];
-  const int64_t giant_slots = (int64_t)hc->gslots;
+  const int64_t giant_slots = (int64_t)hc->giants[0];
   if (giant_slots > 0 && (s = ensure_pool(h, c, giant_slots)) != LOUVAIN_OK) return s;
   MergeArgs<M> a;
   a.g = g; a.Cp = ws.Cp; a.coff = ws.coff; a.cverts = ws.cverts; a.cdeg = ws.cdeg; a.hoff = rs.hoff; a.hend = rs.hend;
@@ -1301,8 +1309,9 @@ louvain_status run_impl(louvain_handle h, Ctx& c, int64_t n, int64_t n_arcs, con
     cudaEventRecord(h->events[e0], c.s);
     const int64_t n_cur = g.n;
     // (a1) pass init: buckets, K' / Sigma' / C' / flags
-    int64_t hb[kNumBuckets + 1], gslots = 0;
-    if ((s = degree_buckets(h, c, g, hb, &gslots)) != LOUVAIN_OK) return s;
+    int64_t hb[kNumBuckets + 1];
+    GiantRows giants;
+    if ((s = degree_buckets(h, c, g, hb, &giants)) != LOUVAIN_OK) return s;
     if (lp == 0) {
       vertex_init<M>(c, st, n_cur, false);
       row_sums<M>(c, g, ws.dperm, hb, st.K, st.Sig, reinterpret_cast<A*>(ws.K0));
@@ -1321,7 +1330,7 @@ louvain_status run_impl(louvain_handle h, Ctx& c, int64_t n, int64_t n_arcs, con
     int64_t moves = 0;
     int32_t ncolours = 0, nrounds = 0, ngraphs = 0;
     float gms = 0.f;
-    if ((s = local_move_phase<M>(h, c, g, hb, gslots, p, lp, tau, &li, &moves, e0 + 2, nullptr, nullptr, 0, &ncolours,
+    if ((s = local_move_phase<M>(h, c, g, hb, giants, p, lp, tau, &li, &moves, e0 + 2, nullptr, nullptr, 0, &ncolours,
                                  &nrounds, &gms, &ngraphs)) != LOUVAIN_OK)
       return s;
     cudaEventRecord(h->events[e0 + 3], c.s);
@@ -1410,8 +1419,9 @@ louvain_status run_impl(louvain_handle h, Ctx& c, int64_t n, int64_t n_arcs, con
   if (!q_done) {
     // (a10) fp32 weights, or no pass ran: Eq. 1 on the input graph
     const int pm = prof_begin(h, c);
-    int64_t hb0[kNumBuckets + 1], gs0 = 0;
-    if ((s = degree_buckets(h, c, g0, hb0, &gs0)) != LOUVAIN_OK) return s;
+    int64_t hb0[kNumBuckets + 1];
+    GiantRows giants0;
+    if ((s = degree_buckets(h, c, g0, hb0, &giants0)) != LOUVAIN_OK) return s;
     modularity_bucketed<M>(c, g0, C, reinterpret_cast<A*>(ws.tot), ws.ctrl, ws.dperm, hb0, ws.gpv);
     prof_end(h, c, kModularity, pm);
   }
@@ -1473,8 +1483,9 @@ louvain_status run_batch_impl(louvain_handle h, Ctx& c, int32_t G, int64_t n, in
   int32_t passes = 0;
   for (int32_t lp = 0; lp < p.max_passes && g.n > 0; lp++) {
     const int64_t n_cur = g.n;
-    int64_t hb[kNumBuckets + 1], gslots = 0;
-    if ((s = degree_buckets(h, c, g, hb, &gslots)) != LOUVAIN_OK) return s;
+    int64_t hb[kNumBuckets + 1];
+    GiantRows giants;
+    if ((s = degree_buckets(h, c, g, hb, &giants)) != LOUVAIN_OK) return s;
     if (lp == 0) {
       vertex_init<M>(c, st, n_cur, false);
       row_sums<M>(c, g, ws.dperm, hb, st.K, st.Sig, reinterpret_cast<A*>(ws.K0));
@@ -1487,7 +1498,7 @@ louvain_status run_batch_impl(louvain_handle h, Ctx& c, int32_t G, int64_t n, in
     }
     int32_t li = 0;
     int64_t moves = 0;
-    if ((s = local_move_phase<M>(h, c, g, hb, gslots, p, lp, tau, &li, &moves, 1, ws.gc, vg, G)) != LOUVAIN_OK)
+    if ((s = local_move_phase<M>(h, c, g, hb, giants, p, lp, tau, &li, &moves, 1, ws.gc, vg, G)) != LOUVAIN_OK)
       return s;
     passes = lp + 1;
     // renumbering, pass tests per graph, dendrogram lookup, next level
@@ -1523,8 +1534,9 @@ louvain_status run_batch_impl(louvain_handle h, Ctx& c, int32_t G, int64_t n, in
   batch_close(c, C, n, ws.vg0, ws.gc, G);
   // (a10) Eq. 1 per graph on the input graphs
   const int pm = prof_begin(h, c);
-  int64_t hb0[kNumBuckets + 1], gs0 = 0;
-  if ((s = degree_buckets(h, c, g0, hb0, &gs0)) != LOUVAIN_OK) return s;
+  int64_t hb0[kNumBuckets + 1];
+  GiantRows giants0;
+  if ((s = degree_buckets(h, c, g0, hb0, &giants0)) != LOUVAIN_OK) return s;
   batch_modularity<M>(c, g0, C, ws.vg0, ws.gc, G, ws.vo, ws.dperm, hb0, st.Sig, reinterpret_cast<A*>(ws.tot), n);
   prof_end(h, c, kModularity, pm);
   const Ctrl* hc = read_ctrl(h, c, &s, "batch modularity");
@@ -2148,15 +2160,16 @@ louvain_status louvain_modularity(louvain_handle h, int64_t n, int64_t n_arcs, c
   const Ctrl* hc = read_ctrl(h, c, &s, "membership range");
   if (!hc) return s;
   if (hc->cnt[5]) return set_err(h, LOUVAIN_ERR_INVALID, "membership id outside [0, n)");
-  int64_t hb[kNumBuckets + 1], gs = 0;
+  int64_t hb[kNumBuckets + 1];
+  GiantRows giants;
   if (fp) {
     GraphView<float> g{n, d_offsets, d_offsets + 1, d_targets, reinterpret_cast<const float*>(d_weights)};
-    if ((s = degree_buckets(h, c, g, hb, &gs)) != LOUVAIN_OK) return s;
+    if ((s = degree_buckets(h, c, g, hb, &giants)) != LOUVAIN_OK) return s;
     modularity_bucketed<FpMode>(c, g, d_membership, reinterpret_cast<double*>(h->ws.tot), h->ws.ctrl, h->ws.dperm, hb,
                                 h->ws.gpv);
   } else {
     GraphView<int32_t> g{n, d_offsets, d_offsets + 1, d_targets, reinterpret_cast<const int32_t*>(d_weights)};
-    if ((s = degree_buckets(h, c, g, hb, &gs)) != LOUVAIN_OK) return s;
+    if ((s = degree_buckets(h, c, g, hb, &giants)) != LOUVAIN_OK) return s;
     modularity_bucketed<IntMode>(c, g, d_membership, reinterpret_cast<long long*>(h->ws.tot), h->ws.ctrl, h->ws.dperm,
                                  hb, h->ws.gpv);
   }
@@ -2195,11 +2208,12 @@ louvain_status louvain_colour(louvain_handle h, int64_t n, int64_t n_arcs, const
   if (!hc) return s;
   if (hc->cnt[5]) return set_err(h, LOUVAIN_ERR_INVALID, "arc target outside [0, n)");
   GraphView<int32_t> g{n, d_offsets, d_offsets + 1, d_targets, nullptr};
-  int64_t hb[kNumBuckets + 1], gslots;
-  if ((s = degree_buckets(h, c, g, hb, &gslots)) != LOUVAIN_OK) return s;
+  int64_t hb[kNumBuckets + 1];
+  GiantRows giants;
+  if ((s = degree_buckets(h, c, g, hb, &giants)) != LOUVAIN_OK) return s;
   JpBuffers jb{h->ws.jrec, h->ws.jl0, h->ws.jl1, h->ws.jlist_cap, h->ws.jused, h->ws.jstate};
   cudaError_t ce;
-  int32_t nc = jp_colour(c, g, h->ws.dperm, hb, seed, pass, d_colour, jb, ctrl, h->pin, &ce);
+  int32_t nc = jp_colour(c, g, h->ws.dperm, hb, seed, pass, d_colour, jb, ctrl, h->pin, &ce, giants.arcs);
   if (ce != cudaSuccess) return cuda_err(h, ce, "colouring");
   if (nc < 0) return colour_failure(h, c);
   *n_colours = nc;
@@ -2241,14 +2255,15 @@ louvain_status louvain_local_move(louvain_handle h, int64_t n, int64_t n_arcs, c
     GraphView<W> g{n, d_offsets, d_offsets + 1, d_targets, reinterpret_cast<const W*>(d_weights)};
     PassState<M> st{reinterpret_cast<A*>(ws.K), reinterpret_cast<A*>(ws.Sig), ws.Cp, ws.flags, ws.csize, ws.mv_from,
                     ws.mv_to, ws.ctrl};
-    int64_t hb[kNumBuckets + 1], gslots;
-    louvain_status r = degree_buckets(h, c, g, hb, &gslots);
+    int64_t hb[kNumBuckets + 1];
+    GiantRows giants;
+    louvain_status r = degree_buckets(h, c, g, hb, &giants);
     if (r != LOUVAIN_OK) return r;
     vertex_init<M>(c, st, n, false);
     row_sums<M>(c, g, ws.dperm, hb, st.K, st.Sig, reinterpret_cast<A*>(ws.K0));
     total_weight<M>(c, st.K, n, ws.ctrl);
     if (!event_at(h, 3)) return set_err(h, LOUVAIN_ERR_CUDA, "event creation failed");
-    r = local_move_phase<M>(h, c, g, hb, gslots, *p, pass, tau, iterations, moves, 3);
+    r = local_move_phase<M>(h, c, g, hb, giants, *p, pass, tau, iterations, moves, 3);
     if (r != LOUVAIN_OK) return r;
     cudaMemcpyAsync(d_cprime, ws.Cp, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c.s);
     if ((r = sync(h, c, "local move end")) == LOUVAIN_OK) pool_done(h);
@@ -2294,8 +2309,9 @@ louvain_status louvain_aggregate(louvain_handle h, int64_t n, int64_t n_arcs, co
     typedef typename M::w_t W;
     GraphView<W> g{n, d_offsets, d_offsets + 1, d_targets, reinterpret_cast<const W*>(d_weights)};
     RowSet& rs = ws.rows[0];
-    int64_t hb[kNumBuckets + 1], gslots;
-    louvain_status r = degree_buckets(h, c, g, hb, &gslots);
+    int64_t hb[kNumBuckets + 1];
+    GiantRows giants;
+    louvain_status r = degree_buckets(h, c, g, hb, &giants);
     if (r != LOUVAIN_OK) return r;
     int64_t cb[kNumBuckets + 1];
     r = aggregate_phase<M>(h, c, g, hb, n_comm, rs, ws.tgA, reinterpret_cast<W*>(ws.wA), cb);

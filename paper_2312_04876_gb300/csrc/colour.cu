@@ -455,7 +455,7 @@ static cudaError_t jp_launch(Scope sc, const Ctx& c, const JpArgs& a, const Pers
 
 int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g, const int32_t* perm, const int64_t* hb, uint64_t seed,
                   int32_t pass, int32_t* colour, const JpBuffers& jb, Ctrl* ctrl, unsigned long long* h_pinned,
-                  cudaError_t* err, Segs seg, int64_t* rounds_out) {
+                  cudaError_t* err, int64_t giant_arcs, Segs seg, int64_t* rounds_out) {
   const int64_t listed = hb[kNumBuckets] - hb[0];
   if (listed < g.n) fill_i32(c, colour, 0, g.n);  // isolated vertices (not listed) get colour 0
   if ((*err = cudaMemsetAsync(jb.state, 0, kJpWords * sizeof(unsigned long long), c.s)) != cudaSuccess) return -1;
@@ -467,12 +467,13 @@ int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g, const int32_t* perm, cons
   a.key = mix64(mix64(seed + gm) + (uint64_t)pass + 2 * gm) + 3 * gm;
   for (int b = 0; b <= kNumBuckets; b++) a.hb[b] = (int32_t)hb[b];
   PersistBar bar{jb.state + kJpBar, c.wait_spins > 0 ? c.wait_spins : kBarrierPolls, 0, 0};
-  // entries a round may hold at most with 8-arc chunks, and the arcs (typical row of each bucket)
-  static const int64_t kChunks[kNumBuckets] = {1, 2, 16, 64, 256, 512, 0}, kArcs[kNumBuckets] = {3, 9, 48, 256, 1024, 3000, 12000};
+  // entries a round may hold at most with 8-arc chunks, and the arcs, about
+  static const int64_t kChunks[kNumBuckets] = {1, 2, 16, 64, 256, 512, 0};
   int64_t chunks = 0, arcs = 0;
   for (int b = 0; b < kNumBuckets; b++) {
     chunks += (hb[b + 1] - hb[b]) * kChunks[b];
-    arcs += (hb[b + 1] - hb[b]) * kArcs[b];
+    const int64_t about = (hb[b + 1] - hb[b]) * kTypicalArcs[b];
+    arcs += b == kNumBuckets - 1 && giant_arcs > about ? giant_arcs : about;
   }
   const bool low = hb[kNumBuckets] == hb[kNumBuckets - 1] && chunks <= jb.list_cap && arcs <= 8 * listed;
   // One block up to ~60,000 arcs, a cluster up to ~500,000 arcs on few vertices (dense super-vertex

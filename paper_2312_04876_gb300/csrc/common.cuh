@@ -49,7 +49,7 @@ struct Ctrl {
   long long acc_i[4];                 // general integer accumulators
   double acc_f[4];                    // general fp accumulators
   double q;                           // last modularity
-  unsigned long long gslots;          // table slots the giant rows of a bucket sort need
+  unsigned long long giants[3];       // giant rows of a bucket sort: table slots they need, arcs, longest
   // algorithmic-traffic counters, summed over a run (reset by the host before each run)
   unsigned long long lm_stat[kNumBuckets][6];  // local move: list entries, vertices processed, arcs
                                                 // scanned, candidates scored, moves, neighbour marks

@@ -87,11 +87,11 @@ struct KeyDesc {
 // left out.  hist must hold nkeys + 1 int64; cursor nkeys int32.  Writes perm and offsets[nkeys+1]
 // (device).
 // max_deg (device, optional) receives the largest row length / deg64 value seen (atomicMax);
-// giant_slots (device, optional) the summed table size of the giant-bucket items, each
-// 2^tbl_log2(min(deg, n_bound), 6, 40).
+// giants (device, optional, three words) of the giant-bucket items the summed table size, each
+// 2^tbl_log2(min(deg, n_bound), 6, 40), the summed length and the largest.
 void bucket_sort(Ctx& c, KeyDesc key_kind, int64_t n, const int64_t* rbeg, const int64_t* rend, const int32_t* colour,
                  const int64_t* deg64, int64_t nkeys, int32_t* perm, int64_t* offsets, int32_t* cursor,
-                 int64_t* tile_tmp, unsigned long long* max_deg, unsigned long long* giant_slots = nullptr,
+                 int64_t* tile_tmp, unsigned long long* max_deg, unsigned long long* giants = nullptr,
                  int64_t n_bound = 0);
 
 // Renumbering (rank among occupied ids): occ[0, n) zeroed then marked from ids[0, m).
@@ -152,6 +152,11 @@ void move_apply(Ctx& c, const PassState<M>& st, const int32_t* list, int64_t cou
 template <class M>
 void move_finish(Ctx& c, Ctrl* ctrl);
 
+// Arcs of a row of each degree bucket, about: the scopes of the persistent launches are chosen by sums of
+// these.  A giant row can be of any length (repeated arcs are accepted, so even on few vertices), so the
+// giants count by their own where that is more.
+constexpr int64_t kTypicalArcs[kNumBuckets] = {3, 9, 48, 256, 1024, 3000, 12000};
+
 // ---------------------------------------------------------------- colour.cu
 struct JpBuffers {
   int4* rec;                  // [n] vertex records
@@ -165,10 +170,10 @@ constexpr int kJpStateWords = 16;
 // Jones-Plassmann colouring of g (self-loops ignored).  Returns the number of colours.
 // -1 on failure: *err, or h_pinned[3..7] = coloured, colours, listed, rounds, guard trips.
 // Synchronises the stream once.
-// In a batched run `seg` makes the priority hash the graph-local id.
+// giant_arcs: arcs in the giant rows.  In a batched run `seg` makes the priority hash the graph-local id.
 int32_t jp_colour(Ctx& c, const GraphView<int32_t>& g_struct, const int32_t* perm, const int64_t* h_bucket_offs,
                   uint64_t seed, int32_t pass, int32_t* colour, const JpBuffers& jb, Ctrl* ctrl,
-                  unsigned long long* h_pinned, cudaError_t* err, Segs seg = Segs(),
+                  unsigned long long* h_pinned, cudaError_t* err, int64_t giant_arcs, Segs seg = Segs(),
                   int64_t* rounds_out = nullptr);
 
 // ---------------------------------------------------------------- aggregate.cu

@@ -223,8 +223,8 @@ constexpr int kSmemKeys = 4096;
 __global__ void __launch_bounds__(kBlock) k_key_hist(KeyDesc kind, int64_t n, const int64_t* rbeg, const int64_t* rend,
                                                      const int32_t* colour, const int64_t* deg64, int64_t nkeys,
                                                      int64_t* hist, unsigned long long* max_deg,
-                                                     unsigned long long* giant_slots, int64_t n_bound) {
-  unsigned long long gs = 0;
+                                                     unsigned long long* giants, int64_t n_bound) {
+  unsigned long long gs = 0, ga = 0, gm = 0;
   __shared__ int32_t sh[kSmemKeys];
   const bool local = nkeys <= kSmemKeys;
   if (local) {
@@ -235,17 +235,29 @@ __global__ void __launch_bounds__(kBlock) k_key_hist(KeyDesc kind, int64_t n, co
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const long long dg = kind.kind == 2 ? deg64[i] : rend[i] - rbeg[i];
     mx = dg > mx ? dg : mx;
-    if (giant_slots && bucket_of(dg, kind.giant_min) == kNumBuckets - 1)
+    if (giants && bucket_of(dg, kind.giant_min) == kNumBuckets - 1) {
       gs += 1ULL << tbl_log2f(dg < n_bound ? dg : n_bound, kind.table_factor, 6, 31);
+      ga += (unsigned long long)dg;
+      gm = (unsigned long long)dg > gm ? (unsigned long long)dg : gm;
+    }
     int k = sort_key(kind, i, rbeg, rend, colour, deg64);
     if (k < 0) continue;
     if (local) atomicAdd(&sh[k], 1);
     else atomicAdd(reinterpret_cast<unsigned long long*>(&hist[k]), 1ULL);
   }
-  if (giant_slots) {
+  if (giants && __any_sync(0xffffffffu, gs != 0)) {
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
-    if ((threadIdx.x & 31) == 0 && gs) atomicAdd(giant_slots, gs);
+    for (int o = 16; o >= 1; o >>= 1) {
+      gs += __shfl_xor_sync(0xffffffffu, gs, o);
+      ga += __shfl_xor_sync(0xffffffffu, ga, o);
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, gm, o);
+      gm = y > gm ? y : gm;
+    }
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(&giants[0], gs);
+      atomicAdd(&giants[1], ga);
+      atomicMax(&giants[2], gm);
+    }
   }
   if (max_deg) {
 #pragma unroll
@@ -314,7 +326,7 @@ constexpr int64_t kSortBlockMax = 8192;
 __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const int64_t* rbeg, const int64_t* rend,
                                                      const int32_t* colour, const int64_t* deg64, int nkeys,
                                                      int32_t* perm, int64_t* offsets, unsigned long long* max_deg,
-                                                     unsigned long long* giant_slots, int64_t n_bound) {
+                                                     unsigned long long* giants, int64_t n_bound) {
   __shared__ int32_t sh[kSmemKeys];
   __shared__ int32_t ws[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -322,7 +334,7 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
   int key[R];
   for (int k = threadIdx.x; k < nkeys; k += 1024) sh[k] = 0;
   __syncthreads();
-  unsigned long long gs = 0;
+  unsigned long long gs = 0, ga = 0, gm = 0;
   long long mx = 0;
 #pragma unroll
   for (int r = 0; r < R; r++) {
@@ -331,12 +343,19 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
     if (i >= n) continue;
     const long long dg = kind.kind == 2 ? deg64[i] : rend[i] - rbeg[i];
     mx = dg > mx ? dg : mx;
-    if (giant_slots && bucket_of(dg, kind.giant_min) == kNumBuckets - 1)
+    if (giants && bucket_of(dg, kind.giant_min) == kNumBuckets - 1) {
       gs += 1ULL << tbl_log2f(dg < n_bound ? dg : n_bound, kind.table_factor, 6, 31);
+      ga += (unsigned long long)dg;
+      gm = (unsigned long long)dg > gm ? (unsigned long long)dg : gm;
+    }
     key[r] = sort_key(kind, i, rbeg, rend, colour, deg64);
     if (key[r] >= 0) atomicAdd(&sh[key[r]], 1);
   }
-  if (giant_slots && gs) atomicAdd(giant_slots, gs);
+  if (giants && gs) {
+    atomicAdd(&giants[0], gs);
+    atomicAdd(&giants[1], ga);
+    atomicMax(&giants[2], gm);
+  }
   if (max_deg && mx > 0) atomicMax(max_deg, (unsigned long long)mx);
   __syncthreads();
   // exclusive scan of the counts, 1024 keys a round
@@ -375,13 +394,13 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
 
 void bucket_sort(Ctx& c, KeyDesc key_kind, int64_t n, const int64_t* rbeg, const int64_t* rend, const int32_t* colour,
                  const int64_t* deg64, int64_t nkeys, int32_t* perm, int64_t* offsets, int32_t* cursor,
-                 int64_t* tile_tmp, unsigned long long* max_deg, unsigned long long* giant_slots,
+                 int64_t* tile_tmp, unsigned long long* max_deg, unsigned long long* giants,
                  int64_t n_bound) {
   key_kind.giant_min = c.giant_min;
   key_kind.table_factor = c.table_factor;
   if (n > 0 && n <= kSortBlockMax && nkeys <= kSmemKeys) {
     k_sort_block<<<1, 1024, 0, c.s>>>(key_kind, (int)n, rbeg, rend, colour, deg64, (int)nkeys, perm, offsets, max_deg,
-                                      giant_slots, n_bound);
+                                      giants, n_bound);
     c.launches++;
     return;
   }
@@ -389,7 +408,7 @@ void bucket_sort(Ctx& c, KeyDesc key_kind, int64_t n, const int64_t* rbeg, const
   cudaMemsetAsync(cursor, 0, (size_t)nkeys * sizeof(int32_t), c.s);
   if (n <= 0) return;
   int grid = grid_for(n, kBlock * 16, c.num_sms * 4);
-  k_key_hist<<<grid, kBlock, 0, c.s>>>(key_kind, n, rbeg, rend, colour, deg64, nkeys, offsets, max_deg, giant_slots,
+  k_key_hist<<<grid, kBlock, 0, c.s>>>(key_kind, n, rbeg, rend, colour, deg64, nkeys, offsets, max_deg, giants,
                                        n_bound);
   scan_exclusive_i64(c, offsets, offsets, nkeys, tile_tmp);
   k_key_scatter<<<grid, kBlock, 0, c.s>>>(key_kind, n, rbeg, rend, colour, deg64, nkeys, offsets, cursor, perm);

@@ -82,7 +82,10 @@ typedef struct {
                                     (one multi-block giant pipeline per iteration); 0 = hash classes */
   int32_t lm_blocks_per_sm;      /* grid cap of the local-moving kernels in blocks per SM (0 = 16); the
                                     degree buckets of a class run concurrently, so smaller grids let
-                                    them share the SMs */
+                                    them share the SMs.  Deterministic mode's class steps run in one
+                                    persistent launch of a block per SM at most, which this does not
+                                    change, except classes of over 2 million arcs with hub rows and
+                                    profiled runs */
   int32_t giant_min_degree;      /* rows longer than this take the multi-block giant path; 2048..4096
                                     (0 = 4096: rows of 2049..4096 arcs use one block with a 64 KB table) */
   int32_t fast_classes_later;    /* fast mode: iterations after the first of a pass may run the classes
@@ -108,8 +111,11 @@ typedef struct {
   int32_t table_factor;          /* hash-table slots per key a table may have to hold: 1, 2 or 4
                                     (tables up to full, half full or a quarter full; 0 = 2), for the
                                     shared-memory tables of merging, the giant rows' global tables
-                                    and, twice as many up to their capacity, those of local moving.  Integer-weight results do not depend on it
-                                    (exact sums, ties by id); it trades probe length for memory */
+                                    and, twice as many up to their capacity, those of the local-moving
+                                    kernels (deterministic mode's persistent class steps have tables
+                                    of their own: four slots per arc, two for rows over 4096 arcs).
+                                    Integer-weight results do not depend on it (exact sums, ties by
+                                    id); it trades probe length for memory */
   int32_t fast_sync_small;       /* fast mode on small graphs: 0 = where the input graph -- a batch:
                                     its mean graph -- fits in what the GPU holds in flight (1024
                                     vertices per SM) and rows over 512 arcs hold at most a fifth of
@@ -273,8 +279,10 @@ louvain_status louvain_run_batch(louvain_handle h, int32_t n_graphs, const int64
  * 2049..4096 arcs: the one-block 64 KB table or the multi-block giant path), lm_blocks_per_sm in
  * {16, 4} and compact in {1, 0}; then table_factor 4 against 2 (hash-table sizes) with the best of
  * those -- and writes *p with the fastest setting into *tuned (other fields copied; *best_ms its
- * time).  In deterministic mode every candidate returns the same
- * membership; d_membership (device, n entries) receives the last run's.  Costs 9 x (reps + 1) runs. */
+ * time).  lm_blocks_per_sm 4 is not tried where no run launches a kernel that it bounds
+ * (deterministic mode without classes of over 2 million arcs); it is then 16.  In deterministic mode
+ * every candidate returns the same membership; d_membership (device, n entries) receives the last
+ * run's.  Costs 9 x (reps + 1) runs, or 5 x where the grid cap is left out. */
 louvain_status louvain_autotune(louvain_handle h, int64_t n, int64_t n_arcs, const int64_t* d_offsets,
                                 const int32_t* d_targets, const void* d_weights, louvain_wtype wtype,
                                 const louvain_params* p, void* stream, int32_t* d_membership, int32_t reps,

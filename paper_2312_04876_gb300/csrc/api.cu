@@ -161,6 +161,7 @@ struct louvain_handle_s {
   int32_t step_from = 0;           // step_from on (injected)
   bool refuse_launch = false;      // cluster and cooperative launches count as refused (injected)
   int64_t fail_alloc_in = 0;       // > 0: the fail_alloc_in-th device allocation from now fails (injected)
+  bool lm_grids = false;           // some local moving since this was cleared launched lm_blocks_per_sm's kernels
   bool arcs_host = false;          // params.host_arcs of the current call: arc buffers in host memory
 };
 
@@ -1173,6 +1174,7 @@ louvain_status local_move_phase(louvain_handle h, Ctx& c, const GraphView<typena
   cudaGraphExec_t g_first = nullptr, g_rest = nullptr;
   int64_t l_first = 0, l_rest = 0;
   const bool graphs = !h->prof.on && h->use_graphs;
+  if (!det || !graphs || layout.f > 0) h->lm_grids = true;
   if (det && graphs)
     return sweep_phase<M>(h, c, g, st, first, layout, glist, p, gc, n_graphs, li, moves, ms_graph, graphs_new);
   int32_t n_new = 0;
@@ -1571,8 +1573,8 @@ louvain_status check_graph_args(louvain_handle h, int64_t n, int64_t n_arcs, con
 // ------------------------------------------------------------------ autotuning
 // Candidates of the performance knobs that leave the arithmetic unchanged: the giant-row
 // threshold (which kernel takes rows of 2049..4096 arcs), the local-move grid cap and super-graph
-// compaction (every combination), then the hash-table sizing (4 slots per key instead of 2) with
-// the best of those.  Each is timed by full runs (device time, best of `reps`) after one untimed run
+// compaction (every combination; the grid cap only where a run launches kernels that have one), then the
+// hash-table sizing (4 slots per key instead of 2) with the best of those.  Each is timed by full runs (device time, best of `reps`) after one untimed run
 // that builds its iteration graphs and buffers, as a run in steady use finds them; the fastest wins.
 template <class RunFn>
 static louvain_status autotune_impl(louvain_handle h, const louvain_params* p, int32_t reps, RunFn run,
@@ -1597,9 +1599,11 @@ static louvain_status autotune_impl(louvain_handle h, const louvain_params* p, i
     return LOUVAIN_OK;
   };
   louvain_status s;
+  h->lm_grids = false;
   for (int32_t gm : kGiant)
     for (int32_t gr : kGrid)
       for (int32_t cp : kCompact) {
+        if (gr != kGrid[0] && !h->lm_grids) continue;  // every trial so far ran persistent class steps alone
         louvain_params q = *p;
         q.giant_min_degree = gm;
         q.lm_blocks_per_sm = gr;

@@ -506,7 +506,9 @@ __device__ __forceinline__ bool pool_put(bool in, int32_t* kv, int lg, int32_t k
   int32_t k[4] = {0, 0, 0, 0};
   bool left = in, load = in;
   unsigned from = 0;  // slots of the bucket, in that order, already found taken
-  for (unsigned p = 0; __any_sync(0xffffffffu, left) && p <= mask + 8; p++) {  // (a bucket takes at most 5 rounds)
+  // a bucket takes at most five rounds: four claims lost to other keys, and one that finds none left
+  const unsigned rounds = 5 * ((mask + 1) / 4);
+  for (unsigned p = 0; __any_sync(0xffffffffu, left) && p < rounds; p++) {
     if (load) {
       const int4 x = __ldcg(reinterpret_cast<const int4*>(kv + 2 * (size_t)s));
       const int4 y = __ldcg(reinterpret_cast<const int4*>(kv + 2 * (size_t)s) + 1);

@@ -84,3 +84,35 @@ def test_kinds_of_rows_of_one_block_do_not_race(rows_a_kind):
 def test_the_replay_sees_a_missing_barrier():
     ops, _, kinds = kernel_ops()
     assert races(ops, [], kinds, 1)
+
+
+def rounds_of_an_insertion(lg):
+    """Rounds that the giant rows' table insertion takes where every claim but the last free slot's is lost to
+    another key: the kernel's probe, one lane, buckets of four slots (as read, `from` on)."""
+    mask = (1 << lg) - 1
+    taken, s, frm, load, view, rounds = set(), 0, 0, True, set(), 0
+    while True:
+        rounds += 1
+        if load:
+            view = set(taken)
+        j = next((t for t in range(frm, 4) if s + t not in view), 4)
+        load = False
+        if j < 4:
+            if s + j not in taken and len(taken) == mask:
+                return rounds
+            taken.add(s + j)  # another key, just before
+            frm = j + 1
+        else:
+            s, frm, load = (s + 4) & mask, 0, True
+
+
+@pytest.mark.parametrize("lg", [6, 7, 10, 14])
+def test_the_pool_insertion_has_rounds_for_its_worst_case(lg):
+    put = between(open(SRC).read(), "bool pool_put(", "\n}\n")
+    limit, = re.findall(r"__any_sync\(0xffffffffu, left\) && p (<=?) ([^;]+); p\+\+", put)
+    names = dict(re.findall(r"const unsigned (\w+) = ([^;]+);", put))
+    bound = limit[1]
+    while bound in names and bound != "mask":
+        bound = names[bound]
+    allowed = eval(bound.replace("/", "//"), {"mask": (1 << lg) - 1}) + (limit[0] == "<=")
+    assert rounds_of_an_insertion(lg) <= allowed

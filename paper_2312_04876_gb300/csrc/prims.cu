@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
   int key[R];
   for (int k = threadIdx.x; k < nkeys; k += 1024) sh[k] = 0;
   __syncthreads();
-  unsigned long long gs = 0, ga = 0, gm = 0;
+  bool giant = false;
   long long mx = 0;
 #pragma unroll
   for (int r = 0; r < R; r++) {
@@ -343,21 +343,12 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
     if (i >= n) continue;
     const long long dg = kind.kind == 2 ? deg64[i] : rend[i] - rbeg[i];
     mx = dg > mx ? dg : mx;
-    if (giants && bucket_of(dg, kind.giant_min) == kNumBuckets - 1) {
-      gs += 1ULL << tbl_log2f(dg < n_bound ? dg : n_bound, kind.table_factor, 6, 31);
-      ga += (unsigned long long)dg;
-      gm = (unsigned long long)dg > gm ? (unsigned long long)dg : gm;
-    }
+    giant |= bucket_of(dg, kind.giant_min) == kNumBuckets - 1;
     key[r] = sort_key(kind, i, rbeg, rend, colour, deg64);
     if (key[r] >= 0) atomicAdd(&sh[key[r]], 1);
   }
-  if (giants && gs) {
-    atomicAdd(&giants[0], gs);
-    atomicAdd(&giants[1], ga);
-    atomicMax(&giants[2], gm);
-  }
   if (max_deg && mx > 0) atomicMax(max_deg, (unsigned long long)mx);
-  __syncthreads();
+  const bool any_giant = __syncthreads_or(giant ? 1 : 0) != 0;
   // exclusive scan of the counts, 1024 keys a round
   int carry = 0;
   for (int base = 0; base < nkeys; base += 1024) {
@@ -390,6 +381,20 @@ __global__ void __launch_bounds__(1024) k_sort_block(KeyDesc kind, int n, const 
 #pragma unroll
   for (int r = 0; r < R; r++)
     if (key[r] >= 0) perm[atomicAdd(&sh[key[r]], 1)] = r * 1024 + (int)threadIdx.x;
+  if (!giants || !any_giant) return;  // (their sums held in the loop above spill)
+  unsigned long long gs = 0, ga = 0, gm = 0;
+  for (int i = threadIdx.x; i < n; i += 1024) {
+    const long long dg = kind.kind == 2 ? deg64[i] : rend[i] - rbeg[i];
+    if (bucket_of(dg, kind.giant_min) != kNumBuckets - 1) continue;
+    gs += 1ULL << tbl_log2f(dg < n_bound ? dg : n_bound, kind.table_factor, 6, 31);
+    ga += (unsigned long long)dg;
+    gm = (unsigned long long)dg > gm ? (unsigned long long)dg : gm;
+  }
+  if (gs) {
+    atomicAdd(&giants[0], gs);
+    atomicAdd(&giants[1], ga);
+    atomicMax(&giants[2], gm);
+  }
 }
 
 void bucket_sort(Ctx& c, KeyDesc key_kind, int64_t n, const int64_t* rbeg, const int64_t* rend, const int32_t* colour,

@@ -229,36 +229,20 @@ __device__ __forceinline__ T group_sum(T v, T* scratch) {
   }
 }
 
-// (score, community) argmax over a group: larger score wins, ties to the smaller community id.
+// (score, community) argmax over a sub-warp group: larger score wins, ties to the smaller community id.
 template <class S>
 __device__ __forceinline__ bool better(S s1, int32_t c1, S s2, int32_t c2) {
   return s1 > s2 || (s1 == s2 && (unsigned)c1 < (unsigned)c2);
 }
 
 template <int G, class S>
-__device__ __forceinline__ void group_argmax(S& s, int32_t& c, S* ss, int32_t* sc) {
-  if (G <= 32) {
-    unsigned m = Grp<G>::mask();
+__device__ __forceinline__ void group_argmax(S& s, int32_t& c) {
+  static_assert(G <= 32, "lanes of a warp");
 #pragma unroll
-    for (int o = G / 2; o >= 1; o >>= 1) {
-      S s2 = __shfl_xor_sync(m, s, o);
-      int32_t c2 = __shfl_xor_sync(m, c, o);
-      if (better(s2, c2, s, c)) { s = s2; c = c2; }
-    }
-  } else {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-      S s2 = __shfl_xor_sync(0xffffffffu, s, o);
-      int32_t c2 = __shfl_xor_sync(0xffffffffu, c, o);
-      if (better(s2, c2, s, c)) { s = s2; c = c2; }
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) { ss[threadIdx.x >> 5] = s; sc[threadIdx.x >> 5] = c; }
-    __syncthreads();
-    s = ss[0]; c = sc[0];
-    for (int w = 1; w < G / 32; w++)
-      if (better(ss[w], sc[w], s, c)) { s = ss[w]; c = sc[w]; }
-    __syncthreads();
+  for (int o = G / 2; o >= 1; o >>= 1) {
+    S s2 = __shfl_xor_sync(Grp<G>::mask(), s, o);
+    int32_t c2 = __shfl_xor_sync(Grp<G>::mask(), c, o);
+    if (better(s2, c2, s, c)) { s = s2; c = c2; }
   }
 }
 
@@ -296,21 +280,6 @@ template <int G>
 __device__ __forceinline__ bool group_any(bool p) {
   if constexpr (G <= 32) return __any_sync(Grp<G>::mask(), p);
   else return __syncthreads_or(p ? 1 : 0) != 0;
-}
-
-// Broadcast lane 0's value to the group.
-template <int G, class T>
-__device__ __forceinline__ T group_bcast(T v, T* scratch) {
-  if (G <= 32) {
-    return __shfl_sync(Grp<G>::mask(), v, 0, G);
-  } else {
-    __syncthreads();
-    if (threadIdx.x == 0) scratch[0] = v;
-    __syncthreads();
-    T r = scratch[0];
-    __syncthreads();
-    return r;
-  }
 }
 
 // ------------------------------------------------------------------ open-addressing table

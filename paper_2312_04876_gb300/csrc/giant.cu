@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kBlock) k_glm_scan(const int32_t* list, int64_
       }
       (void)nb;
     }
-    group_argmax<32>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+    group_argmax<32>(best, bc);
     if (lane == 0) {
       reinterpret_cast<S*>(p.part_s)[q] = best;
       p.part_c[q] = bc;
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kBlock) k_glm_decide(GraphView<typename M::w_t
       const int32_t c = p.part_c[q];
       if (better(s, c, best, bc)) { best = s; bc = c; }
     }
-    group_argmax<32>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+    group_argmax<32>(best, bc);
     if (lane != 0) continue;
     const int32_t i = list[k];
     const int32_t d = st.Cp[i];

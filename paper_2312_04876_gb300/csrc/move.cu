@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(P::T, P::B) lm_kernel(LmArgs<M> a) {
         best = M::score(same, kid, ki, sg, sd, two_m);
         bc = cc[0];
       }
-      group_argmax<G>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+      group_argmax<G>(best, bc);
     } else {
       const int lg = tbl_log2f_fast(deg, 2 * a.tf, 1, LOG);
       const unsigned mask = (1u << lg) - 1;
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(P::T, P::B) lm_kernel(LmArgs<M> a) {
         }
       }
       if constexpr (G < 32) {
-        group_argmax<G>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+        group_argmax<G>(best, bc);
         Grp<G>::sync();  // the table is empty again
       } else {
         __syncwarp();  // for a warp's row: the table is empty again

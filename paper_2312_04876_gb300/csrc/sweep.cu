@@ -299,7 +299,7 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<M>& a, SweepShared<M>&
       best = sweep_score<M>(same, kid, ki, sg, sd, two_m);
       bc = cc[0];
     }
-    group_argmax<4>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+    group_argmax<4>(best, bc);
   } else {
     const int lg = R > 1 ? LOG : tbl_log2f_fast(h.deg, 4, 1, LOG);
     const unsigned size = 1u << lg;
@@ -372,7 +372,7 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<M>& a, SweepShared<M>&
       }
     }
     if constexpr (G < 32) {
-      group_argmax<G>(best, bc, (S*)nullptr, (int32_t*)nullptr);
+      group_argmax<G>(best, bc);
     } else {
       __syncwarp();
       warp_best(best, bc);

@@ -53,7 +53,7 @@ struct Request {
 };
 
 // Upper bound of the device bytes a batched call holds for n vertices and a arcs: the handle's
-// per-vertex state (~220 B), ping-pong super-graph arcs and union targets (20 B/arc), the giant-row
+// per-vertex state (~205 B), ping-pong super-graph arcs and union targets (20 B/arc), the giant-row
 // table pool (<= 40 B per arc in giant rows), plus the lane's union input (offsets, targets,
 // weights, membership).
 size_t estimate_bytes(int64_t n, int64_t a) {
